@@ -22,15 +22,12 @@
 // voxel's channels are contiguous and a 32-channel slice is one 64-byte row.  A
 // cube [N1][N2][N3] is the volume D = N1, H = N2, W = N3.
 //
-// Kernels.  The convolutions are implicit GEMMs on the tensor cores
-// (mma.sync m16n8k16, BF16 in, FP32 accumulate), fed by cp.async gathers:
-//  * conv_fwd_kernel: Y[p, o] = sum_{tap, c} X[p + delta_tap, c] Wt[o, tap, c]:
-//    M = voxels (128 per CTA), N = output channels (32 or 64 per CTA), K = 27
-//    taps x input channels in 32-channel steps; an input may be the channel
-//    concatenation of a same-size tensor and a half-size one read through
-//    nearest upsampling.  Epilogue: bias, ReLU, a ReLU mask (for backward).
-//    The input gradient of a conv is the same kernel with the output gradient
-//    as input and the weights transposed and mirrored, Wb[c, 26 - tap, o].
+// Kernels.
+//  * the convolutions, forward and input gradient, are implicit GEMMs on the
+//    tcgen05 tensor cores (unet_conv.cu); an input may be the channel
+//    concatenation of a half-size tensor read through nearest upsampling and a
+//    same-size one.  The input gradient is the same kernel with the output
+//    gradient as input and the weights transposed and mirrored.
 //  * conv_wgrad_kernel: dW[o, tap, c] = sum_p G[p, o] X[p + delta_tap, c]:
 //    M = output channels, N = 32 input channels of one tap, K = voxels of one
 //    chunk; fragments come from the voxel-major tiles through ldmatrix.trans;
@@ -49,21 +46,17 @@
 #include <new>
 
 #include "s3ttv.h"
+#include "unet_conv.cuh"
 
 namespace {
 
-typedef __nv_bfloat16 bf16;
+using namespace s3ttv_net_detail;
 
 constexpr int kLayers = 10;
 constexpr int kCin[kLayers] = {1, 32, 32, 64, 64, 128, 192, 64, 96, 32};
 constexpr int kCout[kLayers] = {32, 32, 64, 64, 128, 128, 64, 64, 32, 32};
 constexpr int kHeadIn = 32, kHeadOut = 3;
 constexpr long long kMaxVoxels = 1LL << 26;
-
-struct Vol {
-  int B, D, H, W;
-};
-__host__ __device__ inline int nvox(const Vol &g) { return g.B * g.D * g.H * g.W; }
 
 struct LayerTable {
   long long woff[kLayers], boff[kLayers];
@@ -98,12 +91,6 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem, int src
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::); }
 __device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::); }
 
-__device__ __forceinline__ void ldsm_x4(uint32_t r[4], const void *p) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(p);
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(s));
-}
 __device__ __forceinline__ void ldsm_x4_t(uint32_t r[4], const void *p) {
   const unsigned s = (unsigned)__cvta_generic_to_shared(p);
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
@@ -147,173 +134,11 @@ __device__ __forceinline__ void store8(bf16 *p, const float f[8]) {
   *reinterpret_cast<uint4 *>(p) = u;
 }
 
-// ---------------------------------------------------------------- conv forward
-constexpr int kBK = 32;     // input channels per K step
+// ---------------------------------------------------------------- weight gradient
+constexpr int kBK = 32;     // input channels per CTA
 constexpr int kAS = 40;     // shared row stride in bf16 (80 B: ldmatrix rows hit distinct banks)
 constexpr int kStages = 3;  // cp.async pipeline depth
 
-struct ConvArgs {
-  const bf16 *x0;
-  const bf16 *x1;
-  const bf16 *w;       // [cout][27][c1 + c0]
-  const float *bias;   // [cout] or null
-  const bf16 *mask;    // [V][cout] or null: output zeroed where mask <= 0
-  bf16 *y;             // [V][cout]
-  int c0, c1, cout, relu;
-  Vol g;
-};
-
-template <int BM, int BN>
-constexpr int conv_smem_bytes() {
-  return kStages * (BM + BN) * kAS * (int)sizeof(bf16);
-}
-
-// CTA tile BM voxels x BN output channels; (BM / 32) x (BN / 32) warps, each
-// owning a 32 x 32 tile (2 m16 x 4 n8 fragments).  The K loop runs tap by tap
-// and, within a tap, over 32-channel slices of the input; the voxel rows a
-// thread gathers get their neighbour pointers once per tap.
-template <int BM, int BN>
-__global__ void __launch_bounds__((BM / 32) * (BN / 32) * 32) conv_fwd_kernel(ConvArgs a) {
-  constexpr int WN = BN / 32;
-  constexpr int NTH = (BM / 32) * WN * 32;
-  constexpr int RPT = BM * 4 / NTH;  // 16-byte A pieces a thread copies per stage
-  constexpr int AE = BM * kAS, BE = BN * kAS;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  bf16 *As = reinterpret_cast<bf16 *>(smem_raw);
-  bf16 *Bs = As + kStages * AE;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int wm = warp / WN, wn = warp % WN;
-  const int V = nvox(a.g);
-  const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-  const int cin = a.c0 + a.c1, nch = cin / kBK, ksteps = 27 * nch;
-  const int q = tid & 3;
-  // per gathered row: its voxel index, its index in the half-size grid, and a
-  // mask of the volume faces it touches (bit 0/1: z = 0 / D-1, 2/3: y, 4/5: x,
-  // 6: past the last voxel) plus its coordinate parities (bits 8-10: z, y, x)
-  int vi[RPT], li[RPT], rm[RPT];
-  const int D2 = a.g.D >> 1, H2 = a.g.H >> 1, W2 = a.g.W >> 1;
-#pragma unroll
-  for (int i = 0; i < RPT; ++i) {
-    const int p = m0 + (tid >> 2) + i * (NTH / 4);
-    int b, z, y, x;
-    decode(p < V ? p : 0, a.g, b, z, y, x);
-    vi[i] = p;
-    li[i] = ((b * D2 + (z >> 1)) * H2 + (y >> 1)) * W2 + (x >> 1);
-    rm[i] = (z == 0) | (z == a.g.D - 1) << 1 | (y == 0) << 2 | (y == a.g.H - 1) << 3 | (x == 0) << 4 |
-            (x == a.g.W - 1) << 5 | (p >= V) << 6 | (z & 1) << 8 | (y & 1) << 9 | (x & 1) << 10;
-  }
-  // loader state: the tap and slice of the next stage to load; per tap the
-  // faces it may not cross and the neighbour offset in the full-size grid
-  int ltap = -1, lch = nch, forbid = 0, off0 = 0, dz = 0, dy = 0, dx = 0;
-  auto load = [&](int buf) {
-    if (lch == nch) {
-      lch = 0;
-      ++ltap;
-      dz = ltap / 9 - 1;
-      dy = (ltap / 3) % 3 - 1;
-      dx = ltap % 3 - 1;
-      forbid = 64 | (dz < 0) | (dz > 0) << 1 | (dy < 0) << 2 | (dy > 0) << 3 | (dx < 0) << 4 | (dx > 0) << 5;
-      off0 = (dz * a.g.H + dy) * a.g.W + dx;
-    }
-    const int cb = lch * kBK;
-    bf16 *as = As + buf * AE;
-#pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-      const int row = (tid >> 2) + i * (NTH / 4);
-      const bool ok = (rm[i] & forbid) == 0;
-      const bf16 *src;
-      if (cb < a.c1) {
-        // nearest upsampling: the neighbour's half-size cell moves by
-        // floor((parity + d) / 2) along each axis
-        const int oz = (((rm[i] >> 8) & 1) + dz) >> 1, oy = (((rm[i] >> 9) & 1) + dy) >> 1,
-                  ox = (((rm[i] >> 10) & 1) + dx) >> 1;
-        const int n = ok ? li[i] + (oz * H2 + oy) * W2 + ox : 0;
-        src = a.x1 + (size_t)(unsigned)n * a.c1 + cb;
-      } else {
-        const int n = ok ? vi[i] + off0 : 0;
-        src = a.x0 + (size_t)(unsigned)n * a.c0 + (cb - a.c1);
-      }
-      cp_async16(as + row * kAS + q * 8, ok ? src + q * 8 : a.w, ok ? 16 : 0);
-    }
-    bf16 *bs = Bs + buf * BE;
-    const bf16 *wt = a.w + (size_t)ltap * cin + cb;
-    for (int e = tid; e < BN * 4; e += NTH) {
-      const int r = e >> 2, qq = e & 3;
-      cp_async16(bs + r * kAS + qq * 8, wt + (size_t)(n0 + r) * 27 * cin + qq * 8, 16);
-    }
-    ++lch;
-  };
-
-  float acc[2][4][4];
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
-
-#pragma unroll
-  for (int st = 0; st < kStages - 1; ++st) {
-    if (st < ksteps) load(st);
-    cp_async_commit();
-  }
-  for (int ks = 0; ks < ksteps; ++ks) {
-    cp_async_wait1();  // kStages - 2 groups may stay in flight
-    __syncthreads();
-    if (ks + kStages - 1 < ksteps) load((ks + kStages - 1) % kStages);
-    cp_async_commit();
-    const bf16 *as = As + (ks % kStages) * AE, *bs = Bs + (ks % kStages) * BE;
-#pragma unroll
-    for (int kk = 0; kk < kBK; kk += 16) {
-      uint32_t af[2][4], bfr[2][4];
-#pragma unroll
-      for (int mi = 0; mi < 2; ++mi)
-        ldsm_x4(af[mi], as + (wm * 32 + mi * 16 + (lane & 15)) * kAS + kk + (lane >> 4) * 8);
-#pragma unroll
-      for (int nj2 = 0; nj2 < 2; ++nj2)
-        ldsm_x4(bfr[nj2], bs + (wn * 32 + nj2 * 16 + ((lane >> 4) << 3) + (lane & 7)) * kAS + kk +
-                              ((lane >> 3) & 1) * 8);
-#pragma unroll
-      for (int mi = 0; mi < 2; ++mi)
-#pragma unroll
-        for (int nj2 = 0; nj2 < 2; ++nj2) {
-          mma_bf16(acc[mi][2 * nj2], af[mi], bfr[nj2][0], bfr[nj2][1]);
-          mma_bf16(acc[mi][2 * nj2 + 1], af[mi], bfr[nj2][2], bfr[nj2][3]);
-        }
-    }
-  }
-
-  const int gq = lane >> 2, t4 = lane & 3;
-#pragma unroll
-  for (int mi = 0; mi < 2; ++mi)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int row = m0 + wm * 32 + mi * 16 + gq + 8 * h;
-      if (row >= V) continue;
-#pragma unroll
-      for (int nj = 0; nj < 4; ++nj) {
-        const int col = n0 + wn * 32 + nj * 8 + 2 * t4;
-        float v0 = acc[mi][nj][2 * h], v1 = acc[mi][nj][2 * h + 1];
-        if (a.bias) {
-          v0 += a.bias[col];
-          v1 += a.bias[col + 1];
-        }
-        if (a.relu) {
-          v0 = fmaxf(v0, 0.f);
-          v1 = fmaxf(v1, 0.f);
-        }
-        const size_t o = (size_t)row * a.cout + col;
-        if (a.mask) {
-          const __nv_bfloat162 m = *reinterpret_cast<const __nv_bfloat162 *>(a.mask + o);
-          v0 = __bfloat162float(m.x) > 0.f ? v0 : 0.f;
-          v1 = __bfloat162float(m.y) > 0.f ? v1 : 0.f;
-        }
-        *reinterpret_cast<__nv_bfloat162 *>(a.y + o) = __floats2bfloat162_rn(v0, v1);
-      }
-    }
-}
-
-// ---------------------------------------------------------------- weight gradient
 struct WgradArgs {
   const bf16 *g;    // [V][cout] output gradient (ReLU mask applied)
   const bf16 *x0;
@@ -848,9 +673,11 @@ __global__ void adam_kernel(float *theta, const float *g, float *m, float *s, lo
   }
 }
 
-// BF16 copies of the weights: wf in the training layout [o][tap][c], wb as
-// wb[c][26 - tap][o] (the input-gradient conv), hp = the head with its weights
-// rounded to BF16 and its bias in FP32.
+// BF16 copies of the weights: the first layer's as they are ([o][tap]), the
+// others' as the packed images of the forward convolution (wf) and of the
+// input-gradient convolution, whose weight of output c, tap 26 - tap and input o
+// is w[o][tap][c] (wb); hp = the head with its weights rounded to BF16 and its
+// bias in FP32.
 __global__ void pack_kernel(const float *theta, LayerTable t, bf16 *wf, bf16 *wb, float *hp) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < t.total; i += (long long)gridDim.x * blockDim.x) {
     const float x = theta[i];
@@ -862,14 +689,17 @@ __global__ void pack_kernel(const float *theta, LayerTable t, bf16 *wf, bf16 *wb
     int l = 0;
     while (l + 1 < kLayers && i >= t.woff[l + 1]) ++l;
     if (i >= t.boff[l]) continue;  // biases stay FP32 in theta
-    const long long loc = i - t.woff[l];
+    const int loc = (int)(i - t.woff[l]);
     const int ci = t.cin[l], co = t.cout[l];
-    const int o = (int)(loc / (27LL * ci));
-    const int rem = (int)(loc - (long long)o * 27 * ci);
+    const int o = loc / (27 * ci), rem = loc - o * 27 * ci;
     const int tap = rem / ci, c = rem - tap * ci;
     const bf16 h = __float2bfloat16_rn(x);
-    wf[i] = h;
-    wb[t.woff[l] + ((long long)c * 27 + (26 - tap)) * co + o] = h;
+    if (l == 0) {
+      wf[i] = h;
+      continue;
+    }
+    wf[t.woff[l] + conv_pack_index(ci, co, o, tap, c)] = h;
+    wb[t.woff[l] + conv_pack_index(co, ci, c, 26 - tap, o)] = h;
   }
 }
 
@@ -885,6 +715,7 @@ struct s3ttv_net {
   float *theta = nullptr, *grad = nullptr, *m1 = nullptr, *m2 = nullptr, *hp = nullptr;
   bf16 *wf = nullptr, *wb = nullptr;
   double *loss = nullptr;
+  int *err_flag = nullptr;  // host memory the kernels write when a wait of theirs runs out
   long long adam_t = 0;
   bool have_params = false;
   // shape-dependent workspace
@@ -946,16 +777,8 @@ int grid_for(const s3ttv_net *net, long long items, int threads) {
 
 cudaError_t launch_conv(const s3ttv_net *net, const bf16 *x0, int c0, const bf16 *x1, int c1, const bf16 *w,
                         const float *bias, const bf16 *mask, bf16 *y, int cout, bool relu, Vol g) {
-  ConvArgs a{x0, x1, w, bias, mask, y, c0, c1, cout, relu ? 1 : 0, g};
-  const int V = nvox(g);
-  if (cout % 64 == 0) {
-    dim3 grid((V + 127) / 128, cout / 64);
-    conv_fwd_kernel<128, 64><<<grid, 256, conv_smem_bytes<128, 64>(), net->stream>>>(a);
-  } else {
-    dim3 grid((V + 255) / 256, cout / 32);
-    conv_fwd_kernel<256, 32><<<grid, 256, conv_smem_bytes<256, 32>(), net->stream>>>(a);
-  }
-  return cudaGetLastError();
+  ConvArgs a{x0, x1, w, bias, mask, y, c0, c1, cout, relu ? 1 : 0, g, net->err_flag};
+  return conv_launch(a, net->num_sms, net->stream);
 }
 
 cudaError_t launch_wgrad(const s3ttv_net *net, const bf16 *G, int cout, const bf16 *x0, int c0, const bf16 *x1,
@@ -1177,6 +1000,10 @@ int pack(s3ttv_net *net) {
 
 int finish(s3ttv_net *net) {
   NCU(cudaStreamSynchronize(net->stream));
+  if (*(volatile int *)net->err_flag) {
+    *net->err_flag = 0;
+    return nfail(net, S3TTV_ECUDA, "a convolution kernel's wait ran out of time");
+  }
   return S3TTV_OK;
 }
 
@@ -1234,15 +1061,14 @@ int s3ttv_net_create(s3ttv_net **out, int device, void *stream) {
   ok = ok && cudaMalloc(&net->wb, P * sizeof(bf16)) == cudaSuccess;
   ok = ok && cudaMalloc(&net->hp, (kHeadIn * kHeadOut + kHeadOut) * sizeof(float)) == cudaSuccess;
   ok = ok && cudaMalloc(&net->loss, sizeof(double)) == cudaSuccess;
+  ok = ok && cudaHostAlloc(&net->err_flag, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
     s3ttv_net_destroy(net);
     return S3TTV_ENOMEM;
   }
-  if (cudaFuncSetAttribute(conv_fwd_kernel<128, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           conv_smem_bytes<128, 64>()) != cudaSuccess ||
-      cudaFuncSetAttribute(conv_fwd_kernel<256, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           conv_smem_bytes<256, 32>()) != cudaSuccess ||
+  *net->err_flag = 0;
+  if (conv_prepare() != cudaSuccess ||
       cudaFuncSetAttribute(conv_wgrad_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            wgrad_smem_bytes<128>()) != cudaSuccess ||
       cudaFuncSetAttribute(conv_wgrad_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1270,6 +1096,7 @@ void s3ttv_net_destroy(s3ttv_net *net) {
                     net->stage};
     for (void *b : bufs)
       if (b) cudaFree(b);
+    if (net->err_flag) cudaFreeHost(net->err_flag);
     if (net->own_stream) cudaStreamDestroy(net->stream);
   }
   delete net;

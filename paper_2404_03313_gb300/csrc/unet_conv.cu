@@ -1,0 +1,639 @@
+// 3 x 3 x 3 convolution (zero padding, channels-last, BF16 in and out, FP32
+// accumulation) of the warm-start network, forward and input gradient, as an
+// implicit GEMM on the tcgen05 tensor cores: Y[p, n] = sum_{tap, c} X[p + delta_tap, c] W[n, tap, c].
+//
+// A CTA owns a column of the volume, 8 voxels along x (W) by 16 J along y (H),
+// and marches along z (D).  Each plane of the column is copied into shared memory
+// once, with its one-voxel halo, as [c / 8][y][x] pieces of 8 channels (16 bytes):
+// the no-swizzle K-major operand layout, in which an 8-row core matrix is 8
+// voxels of a row of x, the next one is the next y (SBO = one halo row), and a
+// tap's shift in y and x is an offset of the descriptor's start address.  So the
+// 27 neighbours of a voxel cost no copies and no address arithmetic.
+//
+// Plane p serves three output planes: z = p - 1 with the taps dz = +1, z = p with
+// dz = 0, z = p + 1 with dz = -1.  The three have the same A operand for equal
+// (dy, dx), so one tcgen05.mma covers them with N = 3 NT columns: the TMEM
+// accumulators of consecutive z sit in consecutive column slots (a ring; where it
+// wraps, the instruction is split in two) and the B operand holds the three taps'
+// weights one below the other.  That triples the work per byte of A that the
+// tensor cores read from shared memory, which is what bounds M = 128 with N = 32.
+// Every accumulator still sums its products tap by tap and channel by channel.
+//
+// Roles: warps 0-7 read finished accumulators (two warps per quarter of the TMEM
+// lanes, taking turns at blocks of 32 columns), apply bias, ReLU and mask and store
+// BF16; warps 8 and 9 issue the MMAs, one per 128-voxel tile (with one warp for both,
+// issuing took longer than the products: 3500 cycles per plane of 256 voxels and 32
+// channels); warp 10 copies weights (cp.async.bulk, a ring of (dy, dx, channel
+// slice) stages; with 32 input channels all of them once, a CTA keeps its tile of
+// output channels); warps 11-18 copy planes (cp.async with zero fill outside the volume, nearest upsampling
+// by halving the coordinates).  Every wait has a time limit, after which the CTA
+// sets the error flag and ends.
+#include "unet_conv.cuh"
+
+#include <stdint.h>
+
+namespace s3ttv_net_detail {
+namespace {
+
+constexpr int kEpiWarps = 8, kMmaWarp = 8, kWWarp = 10, kLoadWarp0 = 11, kLoadWarps = 8;
+constexpr int kThreads = (kLoadWarp0 + kLoadWarps) * 32;
+constexpr int kTX = 8, kTY = 16;   // a 128-voxel tile: x by y
+constexpr int kPX = kTX + 2;       // halo row
+constexpr int kMaxAStages = 4, kMaxWStages = 16, kMaxSlots = 8;
+constexpr int kTmemCols = 512;
+constexpr int kSmemMax = 227 * 1024 - 2048;
+constexpr int kSmemMin = 120 * 1024;  // one CTA per SM: each takes all of TMEM
+constexpr unsigned long long kWaitNs = 4000000000ull;
+
+// Input channels per weight stage, and whether a CTA keeps all its weights in
+// shared memory (9 stages of 6 or 12 KB at 32 input channels).
+__host__ __device__ constexpr int stage_channels(int cin) { return cin > 96 ? 64 : cin; }
+__host__ __device__ constexpr bool weights_resident(int cin) { return cin == 32; }
+
+struct Plan {
+  int J;               // 128-voxel tiles along y per unit
+  int nt, slots, sh;   // output channels per unit, accumulator slots of the TMEM ring (1 << sh)
+  int lz, nzc;         // output planes per unit, units along z
+  int tx, ty, nn;      // tiles along x, y; channel tiles
+  int units;           // spatial units; each is computed once per channel tile
+  int a_stages, w_stages;
+  int lbo;             // bytes between the 8-channel pieces of a plane
+  int smem;
+};
+
+__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void mbar_init(uint32_t bar, int count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.b32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ unsigned long long now_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  return t;
+}
+// Wait for a barrier's phase; false when the time limit or another role's
+// failure (stop) ends the wait.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *stop) {
+  if (mbar_try(bar, parity)) return true;
+  const unsigned long long t0 = now_ns();
+  while (true) {
+    for (int i = 0; i < 32; ++i)
+      if (mbar_try(bar, parity)) return true;
+    if (*stop) return false;
+    if (now_ns() - t0 > kWaitNs) {
+      *stop = 1;
+      return false;
+    }
+  }
+}
+
+// (.ca: through L1.  With .cg the copies backed up in the load/store unit and held up
+// the epilogue's stores as well: 580 against 470 us for the 192-channel layer.)
+__device__ __forceinline__ void cp16(uint32_t smem, const void *gmem, int bytes) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;\n" ::"r"(smem), "l"(gmem), "r"(bytes));
+}
+__device__ __forceinline__ void bulk_copy(uint32_t smem, const void *gmem, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(smem),
+               "l"(gmem), "r"(bytes), "r"(bar)
+               : "memory");
+}
+// A value that is the same in every lane, as the compiler can see it: operands of
+// tcgen05.mma live in uniform registers, and moving each one there before every
+// instruction cost more than the instruction (130 against 56 cycles at N = 96).
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
+
+// One lane of a converged warp (the same one each time).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.b32 %0, 1, 0, p;\n}\n" : "=r"(r));
+  return r != 0;
+}
+// The operand descriptors come as their low and high words: the high words are
+// constants and only the low ones (start address) move.  add = 0: D = A B, else
+// D += A B.
+__device__ __forceinline__ void mma_f16(uint32_t d, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+                                        uint32_t idesc, uint32_t add = 1u) {
+  asm volatile(
+      "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %6, 0;\n mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}\n" ::"r"(d),
+      "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(add)
+      : "memory");
+}
+__device__ __forceinline__ void mma_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t (&v)[32], uint32_t addr) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,"
+      "%30,%31}, [%32];\n"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
+        "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
+        "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+      : "r"(addr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
+__device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
+
+// No-swizzle K-major operand descriptor.  Low word: start address and the bytes
+// between the two 8-channel halves of a K = 16 step (lbo); high word: the bytes
+// between 8-row groups (sbo) and the descriptor version.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lbo) {
+  return ((lbo >> 4) << 16) | ((addr & 0x3ffffu) >> 4);
+}
+__device__ __forceinline__ uint32_t desc_hi(uint32_t sbo) { return (1u << 14) | (sbo >> 4); }
+
+// 32 bytes (a whole L2 sector) in one store
+__device__ __forceinline__ void st_sector(void *p, const uint32_t *v) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+               "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
+}
+
+// One work unit: an (x, y) column and a chunk of z.
+struct Unit {
+  int b, x0, y0, z0, z1;  // output planes [z0, z1)
+  int p0, p1;                // input planes [p0, p1]
+};
+__device__ __forceinline__ Unit unit_at(int u, const Plan &pl, const Vol &g) {
+  Unit t;
+  t.x0 = (u % pl.tx) * kTX;
+  u /= pl.tx;
+  t.y0 = (u % pl.ty) * kTY * pl.J;
+  u /= pl.ty;
+  t.z0 = (u % pl.nzc) * pl.lz;
+  t.b = u / pl.nzc;
+  t.z1 = min(t.z0 + pl.lz, g.D);
+  t.p0 = max(t.z0 - 1, 0);
+  t.p1 = min(t.z1, g.D - 1);
+  return t;
+}
+
+template <int C0, int C1, int J>
+__global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan pl) {
+  constexpr int CIN = C0 + C1, NQ = CIN / 8;
+  constexpr int CS = stage_channels(CIN), NS = CIN / CS;  // channels per weight stage
+  constexpr bool RES = weights_resident(CIN);
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ __align__(8) uint64_t bars[2 * kMaxAStages + 2 * kMaxWStages + 2 * kMaxSlots + 2];
+  __shared__ __align__(16) float s_bias[192];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_stop;
+  const int tid = threadIdx.x, lane = tid & 31;
+  // broadcasts, so that the compiler knows the role and TMEM address as warp-uniform
+  // and keeps the MMA loop's operands in uniform registers
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const Vol g = a.g;
+  const int NT = pl.nt, S = pl.slots, nt_tile = blockIdx.x % pl.nn;  // this CTA's tile of output channels
+  const int u0 = blockIdx.x / pl.nn, du = gridDim.x / pl.nn;
+  const uint32_t a_bytes = (uint32_t)pl.lbo * NQ, w_bytes = (uint32_t)(CS / 8) * 3 * NT * 16;
+  const uint32_t sA = smem_u32(smem), sW = sA + a_bytes * pl.a_stages;
+  const uint32_t bar0 = smem_u32(bars);
+  auto a_full = [&](int s) { return bar0 + 8u * s; };
+  auto a_empty = [&](int s) { return bar0 + 8u * (kMaxAStages + s); };
+  auto w_full = [&](int s) { return bar0 + 8u * (2 * kMaxAStages + s); };
+  auto w_empty = [&](int s) { return bar0 + 8u * (2 * kMaxAStages + kMaxWStages + s); };
+  auto c_full = [&](int s) { return bar0 + 8u * (2 * kMaxAStages + 2 * kMaxWStages + s); };
+  auto c_empty = [&](int s) { return bar0 + 8u * (2 * kMaxAStages + 2 * kMaxWStages + kMaxSlots + s); };
+  const uint32_t drained = c_empty(kMaxSlots);  // (two) after a failure: the MMAs issued so far are done
+
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&s_tmem)),
+                 "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+  }
+  if (tid == kMmaWarp * 32) {
+    for (int s = 0; s < kMaxAStages; ++s) {
+      mbar_init(a_full(s), kLoadWarps);
+      mbar_init(a_empty(s), J);
+    }
+    for (int s = 0; s < kMaxWStages; ++s) {
+      mbar_init(w_full(s), 1);
+      mbar_init(w_empty(s), J);
+    }
+    for (int s = 0; s < kMaxSlots; ++s) {
+      mbar_init(c_full(s), J);
+      mbar_init(c_empty(s), kEpiWarps);
+    }
+    mbar_init(drained, 1);
+    mbar_init(drained + 8, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    s_stop = 0;
+  }
+  for (int i = tid; i < a.cout; i += kThreads) s_bias[i] = a.bias ? a.bias[i] : 0.f;
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
+  volatile int *stop = &s_stop;
+
+  if (warp < kEpiWarps) {
+    // ---- epilogue: slot k of the ring holds output plane k, k + S, ... of this CTA ----
+    const int quarter = warp & 3, turn = warp >> 2;
+    const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
+    const int row = quarter * 32 + lane, ry = row >> 3, rx = row & 7, nblk = NT / 32;
+    int slot = 0, job = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int u = u0; u < pl.units && ok; u += du) {
+      const Unit t = unit_at(u, pl, g);
+      for (int z = t.z0; z < t.z1; ++z) {
+        ok = __all_sync(0xffffffffu, mbar_wait(c_full(slot), phase, stop));
+        if (!ok) break;
+        fence_after();
+        // this warp's blocks of the tile are first, first + 2, ...; the slot is free
+        // for the next tile as soon as the last one is in registers
+        const int nb = J * nblk, first = (job & 1) ^ turn;
+        job += nb;
+        if (first >= nb) {
+          if (lane == 0) mbar_arrive(c_empty(slot));
+        }
+        for (int e = first; e < nb; e += 2) {
+          const int sub = e / nblk, c0 = (e - sub * nblk) * 32;
+          const int y = t.y0 + sub * kTY + ry, x = t.x0 + rx;
+          const uint32_t col = lane_base + (uint32_t)((sub * S + slot) * NT + c0);
+          uint32_t v[32];
+          tmem_ld32(v, col);
+          if (e + 2 >= nb) {
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(c_empty(slot));
+          }
+          if (y < g.H && x < g.W) {
+            const size_t vox = (((size_t)t.b * g.D + z) * g.H + y) * g.W + x;
+            const int n0 = nt_tile * NT + c0;
+            const size_t o = vox * a.cout + n0;
+            uint32_t ow[16];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const float4 b4 = *reinterpret_cast<const float4 *>(s_bias + n0 + 4 * i);
+              float f[4] = {__uint_as_float(v[4 * i]) + b4.x, __uint_as_float(v[4 * i + 1]) + b4.y,
+                            __uint_as_float(v[4 * i + 2]) + b4.z, __uint_as_float(v[4 * i + 3]) + b4.w};
+              if (a.relu) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) f[j] = fmaxf(f[j], 0.f);
+              }
+              const __nv_bfloat162 h0 = __floats2bfloat162_rn(f[0], f[1]), h1 = __floats2bfloat162_rn(f[2], f[3]);
+              ow[2 * i] = *reinterpret_cast<const uint32_t *>(&h0);
+              ow[2 * i + 1] = *reinterpret_cast<const uint32_t *>(&h1);
+            }
+            if (a.mask) {
+              const uint4 *mp = reinterpret_cast<const uint4 *>(a.mask + o);
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const uint4 m4 = mp[q];
+                const uint32_t mw[4] = {m4.x, m4.y, m4.z, m4.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  const __nv_bfloat162 m = *reinterpret_cast<const __nv_bfloat162 *>(&mw[i]);
+                  ow[4 * q + i] &= (__bfloat162float(m.x) > 0.f ? 0xffffu : 0u) |
+                                   (__bfloat162float(m.y) > 0.f ? 0xffff0000u : 0u);
+                }
+              }
+            }
+            st_sector(a.y + o, ow);
+            st_sector(a.y + o + 16, ow + 8);
+          }
+          __syncwarp();
+        }
+        if (++slot == S) {
+          slot = 0;
+          phase ^= 1;
+        }
+      }
+    }
+  } else if (warp < kMmaWarp + 2) {
+    // ---- MMA issue: the whole warp runs the (uniform) loop, one lane issues ----
+    if (warp - kMmaWarp < J) {
+      const int sub = warp - kMmaWarp;  // this warp's 128-voxel tile
+      const uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | (8u << 24);  // F32 <- BF16 x BF16, M = 128
+      const uint32_t id0 = idesc0 | ((uint32_t)(NT >> 3) << 17);
+      const uint32_t b_lbo = 3u * NT * 16, ahi = desc_hi(kPX * 16), bhi = desc_hi(128);
+      const uint32_t ak = 2u * pl.lbo >> 4, bk = 2u * b_lbo >> 4;  // descriptor steps of 16 channels
+      const uint32_t wstep = w_bytes >> 4;                          // and of a weight stage
+      const uint32_t dsub = tmem + (uint32_t)(sub * S * NT);       // the tile's accumulator ring
+      const bool issue = elect_one();
+      int as = 0, ws = 0, slot0 = 0;        // slot0: the slot of the unit's first output plane
+      uint32_t aph = 0, wph = 0, cph = 1;   // cph: the parity to wait for in the ring turn slot0 is in
+      bool ok = true;
+      if (RES)
+        for (int st = 0; st < 9; ++st) mbar_wait(w_full(st), 0, stop);
+      for (int u = u0; u < pl.units && ok; u += du) {
+        const Unit t = unit_at(u, pl, g);
+        for (int p = t.p0; p <= t.p1; ++p) {
+          const int zlo = max(p - 1, t.z0), zhi = min(p + 1, t.z1 - 1), n = zhi - zlo + 1;
+          bool got = true;
+          for (int z = zlo; z <= zhi; ++z) {
+            if (p != max(z - 1, 0)) continue;  // not the first plane that adds into z
+            // c_empty(s) completes its phase k - 1 when the slot is free for its k-th use
+            const int k = slot0 + (z - t.z0);
+            got = mbar_wait(c_empty(k & (S - 1)), cph ^ (uint32_t)((k >> pl.sh) & 1), stop) && got;
+          }
+          got = mbar_wait(a_full(as), aph, stop) && got;
+          ok = __all_sync(0xffffffffu, got);
+          if (!ok) break;
+          fence_after();
+          const int s0 = (slot0 + zlo - t.z0) & (S - 1), n1 = min(n, S - s0);
+          // (uniform() tells the compiler what it cannot see through the divisions)
+          const bool wrap = uniform(n1 < n ? 1u : 0u) != 0u;
+          const uint32_t id1 = uniform(idesc0 | ((uint32_t)(n1 * NT >> 3) << 17));
+          const uint32_t id2 = uniform(idesc0 | ((uint32_t)((n - n1) * NT >> 3) << 17));
+          const uint32_t alo = uniform(desc_lo(sA + a_bytes * as + (uint32_t)(sub * kTY * kPX) * 16, pl.lbo));
+          // rows of B: the lowest output plane's block first (block 0 is dz = +1)
+          const uint32_t blo0 = uniform(desc_lo(sW + (uint32_t)((zlo - (p - 1)) * NT) * 16, b_lbo));
+          const uint32_t d1 = uniform(dsub + (uint32_t)(s0 * NT)), bw = uniform((uint32_t)(n1 * NT));
+          uint32_t tap = alo;  // the A descriptor of the tap's shift in y and x
+          // (rolled: straight-line code for nine taps outruns the instruction cache)
+#pragma unroll 1
+          for (int yx = 0; yx < 9; ++yx) {
+#pragma unroll
+            for (int sl = 0; sl < NS; ++sl) {
+              if (!RES) mbar_wait(w_full(ws), wph, stop);  // (a wait that fails shows at the next plane)
+              const uint32_t blo = RES ? blo0 + wstep * yx : uniform(blo0 + wstep * ws);
+              const uint32_t a0 = tap + (uint32_t)(sl * (CS / 16)) * ak;
+              if (issue) {
+                const bool start = sl == 0 && yx == 0;
+                if (start)
+                  // the plane's first step, output plane by output plane: one that no
+                  // plane has added into yet is written instead of added to
+                  for (int i = 0; i < n; ++i)
+                    mma_f16(dsub + (uint32_t)(((s0 + i) & (S - 1)) * NT), a0, ahi, blo + i * NT, bhi, id0,
+                            p == max(zlo + i - 1, 0) ? 0u : 1u);
+#pragma unroll
+                for (int kk = 0; kk < CS / 16; ++kk)
+                  if (kk > 0 || !start) mma_f16(d1, a0 + kk * ak, ahi, blo + kk * bk, bhi, id1);
+                if (wrap) {
+#pragma unroll
+                  for (int kk = 0; kk < CS / 16; ++kk)
+                    if (kk > 0 || !start) mma_f16(dsub, a0 + kk * ak, ahi, blo + kk * bk + bw, bhi, id2);
+                }
+                if (!RES) mma_commit(w_empty(ws));
+              }
+              __syncwarp();
+              if (!RES && ++ws == pl.w_stages) {
+                ws = 0;
+                wph ^= 1;
+              }
+            }
+            tap += yx % 3 == 2 ? kPX - 2 : 1;
+          }
+          if (issue) {
+            mma_commit(a_empty(as));
+            // the planes that p completes: p - 1, and p itself at the volume's end
+            for (int z = zlo; z <= zhi; ++z)
+              if (min(z + 1, g.D - 1) == p) mma_commit(c_full((slot0 + z - t.z0) & (S - 1)));
+          }
+          __syncwarp();
+          if (++as == pl.a_stages) {
+            as = 0;
+            aph ^= 1;
+          }
+        }
+        const int k = slot0 + (t.z1 - t.z0);
+        cph ^= (uint32_t)((k >> pl.sh) & 1);
+        slot0 = k & (S - 1);
+      }
+      if (!ok && issue) {  // drain what was issued before TMEM is given back
+        mma_commit(drained + 8u * sub);
+        const unsigned long long t0 = now_ns();
+        while (!mbar_try(drained + 8u * sub, 0) && now_ns() - t0 < kWaitNs) {
+        }
+      }
+    }
+  } else if (warp == kWWarp) {
+    if (lane == 0) {
+      // ---- weight copies ----
+      int ws = 0;
+      uint32_t ph = 1;
+      bool ok = true;
+      unsigned issued = 0;
+      auto stage_src = [&](int yx, int sl) {
+        return a.w + (((size_t)(nt_tile * 9 + yx) * NQ + sl * (CS / 8)) * 3) * NT * 8;
+      };
+      if (RES) {
+        for (int st = 0; st < 9 * NS; ++st) {
+          mbar_expect(w_full(st), w_bytes);
+          bulk_copy(sW + w_bytes * st, stage_src(st / NS, st % NS), w_bytes, w_full(st));
+          ++issued;
+        }
+      } else {
+        for (int u = u0; u < pl.units && ok; u += du) {
+          const Unit t = unit_at(u, pl, g);
+          for (int p = t.p0; p <= t.p1 && ok; ++p)
+            for (int st = 0; st < 9 * NS; ++st) {
+              if (!(ok = mbar_wait(w_empty(ws), ph, stop))) break;
+              mbar_expect(w_full(ws), w_bytes);
+              bulk_copy(sW + w_bytes * ws, stage_src(st / NS, st % NS), w_bytes, w_full(ws));
+              ++issued;
+              if (++ws == pl.w_stages) {
+                ws = 0;
+                ph ^= 1;
+              }
+            }
+        }
+      }
+      if (RES || !ok) {  // copies in flight land before the CTA ends
+        const unsigned first = issued > (unsigned)pl.w_stages ? issued - pl.w_stages : 0u;
+        const unsigned long long t0 = now_ns();
+        for (unsigned i = first; i < issued; ++i)
+          while (!mbar_try(w_full(i % pl.w_stages), (i / pl.w_stages) & 1) && now_ns() - t0 < kWaitNs) {
+          }
+      }
+    }
+  } else {
+    // ---- plane copies ----
+    // A thread keeps its 8-channel piece q and its NI voxels of the plane, whose
+    // offsets (-1 outside the volume) it computes once per unit.
+    constexpr int LT = (kLoadWarps * 32) / NQ * NQ, VS = LT / NQ, NV = kPX * (kTY * J + 2), NI = (NV + VS - 1) / VS;
+    const int lt = tid - kLoadWarp0 * 32, q = lt % NQ, v0 = lt < LT ? lt / NQ : NV;
+    const bool half = C1 && q < C1 / 8;  // this piece comes from the half-size input
+    const int hs = half ? 1 : 0, C = half ? C1 : C0, Hs = g.H >> hs, Ws = g.W >> hs, Ds = g.D >> hs;
+    const bf16 *base = half ? a.x1 + q * 8 : a.x0 + (q * 8 - C1);
+    auto landed = [&](int s) {  // this warp's copies into stage s are visible to the tensor cores
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(a_full(s));
+    };
+    int as = 0, prev = -1;  // prev: a stage whose copies are in flight
+    uint32_t ph = 1;
+    bool ok = true;
+    for (int u = u0; u < pl.units && ok; u += du) {
+      const Unit t = unit_at(u, pl, g);
+      int off[NI];
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        const int v = v0 + i * VS, vy = v / kPX, vx = v - vy * kPX;
+        const int y = t.y0 + vy - 1, x = t.x0 + vx - 1;
+        const bool in = (unsigned)y < (unsigned)g.H && (unsigned)x < (unsigned)g.W;
+        off[i] = in ? ((y >> hs) * Ws + (x >> hs)) * C : -1;
+      }
+      for (int p = t.p0; p <= t.p1; ++p) {
+        ok = __all_sync(0xffffffffu, mbar_wait(a_empty(as), ph, stop));
+        if (!ok) break;
+        const uint32_t dst = sA + a_bytes * as + (uint32_t)q * pl.lbo + (uint32_t)v0 * 16;
+        const bf16 *plane = base + ((size_t)t.b * Ds + (p >> hs)) * Hs * Ws * C;
+#pragma unroll
+        for (int i = 0; i < NI; ++i)
+          if (lt < LT && ((i + 1) * VS <= NV || v0 + i * VS < NV))
+            cp16(dst + (uint32_t)(i * VS) * 16, plane + max(off[i], 0), off[i] >= 0 ? 16 : 0);
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+        // With three stages or more, the next plane's copies are issued before this one's
+        // are waited for (with two, their stage is the one the tensor cores are reading).
+        if (prev >= 0) {
+          asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+          landed(prev);
+        }
+        prev = as;
+        if (pl.a_stages < 3) {
+          asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+          landed(prev);
+          prev = -1;
+        }
+        if (++as == pl.a_stages) {
+          as = 0;
+          ph ^= 1;
+        }
+      }
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    if (prev >= 0) landed(prev);
+  }
+  __syncwarp();
+  fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTmemCols));
+  }
+  if (tid == 0 && *stop) *reinterpret_cast<volatile int *>(a.err) = 1;
+}
+
+// Tensor-core cycles of one plane that serves n output planes (per 16-channel
+// step, 128-voxel tile and (dy, dx)): the products at N / 2 cycles for M = 128,
+// K = 16, or the operands' 128-byte shared-memory reads, whichever is longer.
+double step_cycles(int n, int nt) {
+  const double products = 0.5 * n * nt, reads = 32.0 + 0.25 * n * nt;
+  return products > reads ? products : reads;
+}
+
+bool fit(Plan &pl, int cin) {
+  const int nq = cin / 8, cs = stage_channels(cin), nst = 9 * (cin / cs);
+  const int nvp = kPX * (kTY * pl.J + 2);
+  // 16-byte pieces of 8 consecutive lanes fall into different banks: 4 pieces of
+  // 2 voxels (32 channels) or the 8 and more pieces of one voxel
+  const int want = nq == 4 ? 2 : 1;
+  pl.lbo = (nvp + ((want - nvp % 8) + 8) % 8) * 16;
+  const int ab = pl.lbo * nq, wb = cs / 8 * 3 * pl.nt * 16;
+  if (weights_resident(cin)) {
+    pl.w_stages = nst;
+    pl.a_stages = 2;
+  } else {
+    pl.a_stages = 2 * ab + 2 * wb <= kSmemMax ? 2 : 1;
+    pl.w_stages = (kSmemMax - pl.a_stages * ab) / wb;
+    if (pl.w_stages > 8) pl.w_stages = 8;
+    if (pl.w_stages < 2) return false;
+  }
+  if (pl.w_stages > kMaxWStages || pl.a_stages * ab + pl.w_stages * wb > kSmemMax) return false;
+  while (pl.a_stages < kMaxAStages && (pl.a_stages + 1) * ab + pl.w_stages * wb <= kSmemMax) ++pl.a_stages;
+  pl.smem = pl.a_stages * ab + pl.w_stages * wb;
+  if (pl.smem < kSmemMin) pl.smem = kSmemMin;
+  return true;
+}
+
+// The split of the volume into work units: tiles along y per unit and planes per
+// unit, by the tensor-core time of the busiest CTA (a plane at either end of a
+// unit serves one or two output planes instead of three, so longer units cost
+// less, but the units have to fill the SMs).
+bool make_plan(const ConvArgs &a, int num_sms, Plan *best) {
+  const int cin = a.c0 + a.c1;
+  double best_cost = 1e300;
+  for (int J = 1; J <= 2; ++J) {
+    if (J == 2 && a.g.H <= kTY) continue;
+    Plan pl;
+    pl.J = J;
+    pl.nt = conv_tile_n(a.cout);
+    pl.nn = a.cout / pl.nt;
+    pl.sh = J * pl.nt > 64 ? 2 : 3;  // 4 slots of 2 x 64 columns, else 8
+    pl.slots = 1 << pl.sh;
+    pl.tx = (a.g.W + kTX - 1) / kTX;
+    pl.ty = (a.g.H + kTY * J - 1) / (kTY * J);
+    if (!fit(pl, cin)) continue;
+    const double steps = 9.0 * (cin / 16) * J;
+    const double c1 = step_cycles(1, pl.nt), c2 = step_cycles(2, pl.nt), c3 = step_cycles(3, pl.nt);
+    for (int lz = 1; lz <= a.g.D; lz = lz < 8 ? lz + 1 : lz + (lz + 3) / 4) {
+      pl.lz = lz;
+      pl.nzc = (a.g.D + lz - 1) / lz;
+      const long long units = (long long)a.g.B * pl.nzc * pl.ty * pl.tx;
+      if (units > (1 << 30)) continue;
+      pl.units = (int)units;
+      const long long ctas = num_sms > pl.nn ? num_sms / pl.nn : 1, waves = (units + ctas - 1) / ctas;
+      const double unit = lz == 1 ? 3 * c1 : 2 * c1 + 2 * c2 + (lz - 2) * c3;
+      const double cost = waves * (steps * unit + 250.0 * (lz + 2) + 1500.0);
+      if (cost < best_cost) {
+        best_cost = cost;
+        *best = pl;
+      }
+    }
+  }
+  return best_cost < 1e300;
+}
+
+template <int C0, int C1>
+cudaError_t launch(const ConvArgs &a, const Plan &pl, int num_sms, cudaStream_t stream) {
+  const int ctas = num_sms > pl.nn ? num_sms / pl.nn : 1, grid = pl.nn * (pl.units < ctas ? pl.units : ctas);
+  if (pl.J == 2)
+    conv_tc_kernel<C0, C1, 2><<<grid, kThreads, pl.smem, stream>>>(a, pl);
+  else
+    conv_tc_kernel<C0, C1, 1><<<grid, kThreads, pl.smem, stream>>>(a, pl);
+  return cudaGetLastError();
+}
+
+template <int C0, int C1>
+cudaError_t prepare() {
+  const cudaError_t e = cudaFuncSetAttribute(conv_tc_kernel<C0, C1, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kSmemMax);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(conv_tc_kernel<C0, C1, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+}
+
+}  // namespace
+
+cudaError_t conv_prepare() {
+  cudaError_t e = prepare<32, 0>();
+  if (e == cudaSuccess) e = prepare<64, 0>();
+  if (e == cudaSuccess) e = prepare<128, 0>();
+  if (e == cudaSuccess) e = prepare<64, 128>();
+  if (e == cudaSuccess) e = prepare<32, 64>();
+  return e;
+}
+
+cudaError_t conv_launch(const ConvArgs &a, int num_sms, cudaStream_t stream) {
+  Plan pl;
+  if (a.cout % 32 || a.cout > 192 || !make_plan(a, num_sms, &pl)) return cudaErrorInvalidValue;
+  if (a.c0 == 32 && a.c1 == 0) return launch<32, 0>(a, pl, num_sms, stream);
+  if (a.c0 == 64 && a.c1 == 0) return launch<64, 0>(a, pl, num_sms, stream);
+  if (a.c0 == 128 && a.c1 == 0) return launch<128, 0>(a, pl, num_sms, stream);
+  if (a.c0 == 64 && a.c1 == 128) return launch<64, 128>(a, pl, num_sms, stream);
+  if (a.c0 == 32 && a.c1 == 64) return launch<32, 64>(a, pl, num_sms, stream);
+  return cudaErrorInvalidValue;
+}
+
+}  // namespace s3ttv_net_detail
