@@ -1782,7 +1782,7 @@ int s3ttv_quality(s3ttv_ctx *ctx, const float *u, const float *ref, int N1, int 
   CU(cudaMemsetAsync(ctx->macc, 0, sizeof(double) * (2 * N3 + 1), ctx->stream));
   const int grid = ctx->num_sms * 8;
   if (mpsnr) CU(launch_band_sqerr(du, dr, P, N3, ctx->macc, grid, ctx->stream));
-  if (mssim) CU(launch_ssim(du, dr, N1, N2, N3, b0, nb, ctx->macc + N3, grid, ctx->stream));
+  if (mssim) CU(launch_ssim(du, dr, N1, N2, N3, b0, nb, ctx->macc + N3, ctx->num_sms, ctx->stream));
   if (sam_mean || sam_map) CU(launch_sam(du, dr, P, N3, dmap, ctx->macc + 2 * N3, grid, ctx->stream));
   if (sam_map && !md)
     CU(cudaMemcpyAsync(sam_map, dmap, sizeof(float) * P, cudaMemcpyDeviceToHost, ctx->stream));

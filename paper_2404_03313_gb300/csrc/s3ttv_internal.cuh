@@ -239,7 +239,7 @@ cudaError_t launch_band_sqerr(const float *u, const float *ref, long long P, int
 cudaError_t launch_sam(const float *u, const float *ref, long long P, int N3, float *map, double *sum, int grid,
                        cudaStream_t st);
 cudaError_t launch_ssim(const float *u, const float *ref, int N1, int N2, int N3, int b0, int nb, double *out,
-                        int grid, cudaStream_t st);
+                        int num_sms, cudaStream_t st);
 size_t objective_smem_bytes(int k, int stacked);  // rows: k^2 or 2k^2
 cudaError_t launch_objective(const float *u, int N1, int N2, int N3, int k, int stacked, int open_s,
                              int first_order, double *out, unsigned *nonconv, int grid, cudaStream_t st,
