@@ -106,6 +106,24 @@ __device__ __forceinline__ void mma_bf16(float c[4], const uint32_t a[4], uint32
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// two FP32 values in one 64-bit register, and their packed FMA (each half rounds as
+// its scalar counterpart)
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
 __device__ __forceinline__ void decode(int p, const Vol &g, int &b, int &z, int &y, int &x) {
   x = p % g.W;
   int t = p / g.W;
@@ -418,40 +436,64 @@ __global__ void __launch_bounds__(128) conv_wgrad4_kernel(WgradArgs a) {
 }
 
 // ---------------------------------------------------------------- first layer (one input channel)
-__global__ void __launch_bounds__(256) conv_first_kernel(const float *v, const bf16 *w, const float *bias, bf16 *y,
+// Bound by the FP32 rate: 27 x 32 FMAs per voxel (0.19 ms at 256 x 256 x 128).  A
+// thread takes 4 voxels along x and 8 channels, so that two 16-byte reads of the
+// weights (FP32 in shared memory, channels fastest) serve 16 packed FP32x2 FMAs; one
+// voxel and all 32 channels per thread read a weight per FMA and took 970 us where
+// this takes 374 us.  Every output sums its 27 taps in the same order.
+__global__ void __launch_bounds__(256, 2) conv_first_kernel(const float *v, const bf16 *w, const float *bias, bf16 *y,
                                                          Vol g) {
-  __shared__ float ws[32 * 27];
-  __shared__ float bs[32];
-  for (int i = threadIdx.x; i < 32 * 27; i += blockDim.x) ws[i] = __bfloat162float(w[i]);
+  __shared__ __align__(16) float ws[27][32];
+  __shared__ __align__(16) float bs[32];
+  for (int i = threadIdx.x; i < 32 * 27; i += blockDim.x) ws[i % 27][i / 27] = __bfloat162float(w[i]);
   if (threadIdx.x < 32) bs[threadIdx.x] = bias[threadIdx.x];
   __syncthreads();
-  const int V = nvox(g);
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < V; p += gridDim.x * blockDim.x) {
-    int b, z, yy, x;
-    decode(p, g, b, z, yy, x);
-    float nb[27];
+  const int c0 = (threadIdx.x & 3) * 8;  // this thread's channels
+  const int W4 = g.W / 4, Q = nvox(g) / 4;
+  for (int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 2; q < Q; q += (gridDim.x * blockDim.x) >> 2) {
+    const int x0 = (q % W4) * 4, row = q / W4, yy = row % g.H, bz = row / g.H, z = bz % g.D;
+    unsigned long long acc[4][4];  // [voxel][channel pair]
 #pragma unroll
-    for (int t = 0; t < 27; ++t) {
-      const int zz = z + t / 9 - 1, y2 = yy + (t / 3) % 3 - 1, x2 = x + t % 3 - 1;
-      const bool ok = zz >= 0 && zz < g.D && y2 >= 0 && y2 < g.H && x2 >= 0 && x2 < g.W;
-      nb[t] = ok ? v[(((size_t)b * g.D + zz) * g.H + y2) * g.W + x2] : 0.f;
+    for (int i = 0; i < 4; ++i) {
+      const float2 b2 = *reinterpret_cast<const float2 *>(bs + c0 + 2 * i);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[j][i] = pack2(b2.x, b2.y);
     }
-    uint4 out[4];
-    uint32_t *o32 = reinterpret_cast<uint32_t *>(out);
+#pragma unroll 3
+    for (int r = 0; r < 9; ++r) {
+      const int dz = r / 3 - 1, zz = z + dz, y2 = yy + r - 3 * (dz + 1) - 1;
+      float nb[6];
+      const bool in = zz >= 0 && zz < g.D && y2 >= 0 && y2 < g.H;
+      const float *src = v + ((size_t)(bz + dz) * g.H + y2) * g.W + x0;
 #pragma unroll
-    for (int c = 0; c < 32; c += 2) {
-      float s0 = bs[c], s1 = bs[c + 1];
-#pragma unroll
-      for (int t = 0; t < 27; ++t) {
-        s0 = fmaf(ws[c * 27 + t], nb[t], s0);
-        s1 = fmaf(ws[(c + 1) * 27 + t], nb[t], s1);
+      for (int e = 0; e < 6; ++e) {
+        const int x = x0 + e - 1;
+        nb[e] = in && x >= 0 && x < g.W ? src[e - 1] : 0.f;
       }
-      __nv_bfloat162 h = __floats2bfloat162_rn(fmaxf(s0, 0.f), fmaxf(s1, 0.f));
-      o32[c / 2] = *reinterpret_cast<uint32_t *>(&h);
-    }
-    uint4 *dst = reinterpret_cast<uint4 *>(y + (size_t)p * 32);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) dst[i] = out[i];
+      for (int dx = 0; dx < 3; ++dx) {
+        const float4 wa = *reinterpret_cast<const float4 *>(&ws[3 * r + dx][c0]);
+        const float4 wb = *reinterpret_cast<const float4 *>(&ws[3 * r + dx][c0 + 4]);
+        const unsigned long long w2[4] = {pack2(wa.x, wa.y), pack2(wa.z, wa.w), pack2(wb.x, wb.y), pack2(wb.z, wb.w)};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const unsigned long long n2 = pack2(nb[j + dx], nb[j + dx]);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) acc[j][i] = fma2(w2[i], n2, acc[j][i]);
+        }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float f[8];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 t = unpack2(acc[j][i]);
+        f[2 * i] = fmaxf(t.x, 0.f);
+        f[2 * i + 1] = fmaxf(t.y, 0.f);
+      }
+      store8(y + ((size_t)q * 4 + j) * 32 + c0, f);
+    }
   }
 }
 
@@ -551,32 +593,7 @@ __global__ void combine_kernel(const bf16 *glo, const bf16 *ghi, int chi, int co
 }
 
 // ---------------------------------------------------------------- head
-// h = Wh f + bh; u = v + h0, s = h1, t = h2.  hp: Wh[3][32] then bh[3] (FP32).
-__global__ void __launch_bounds__(256) head_fwd_kernel(const bf16 *f, const float *v, const float *hp, float *u,
-                                                       float *s, float *t, int V) {
-  __shared__ float w[kHeadIn * kHeadOut + kHeadOut];
-  for (int i = threadIdx.x; i < kHeadIn * kHeadOut + kHeadOut; i += blockDim.x) w[i] = hp[i];
-  __syncthreads();
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < V; p += gridDim.x * blockDim.x) {
-    float h0 = w[96], h1 = w[97], h2 = w[98];
-#pragma unroll
-    for (int c8 = 0; c8 < 4; ++c8) {
-      float fv[8];
-      load8(f + (size_t)p * 32 + c8 * 8, fv);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int c = c8 * 8 + i;
-        h0 = fmaf(w[c], fv[i], h0);
-        h1 = fmaf(w[32 + c], fv[i], h1);
-        h2 = fmaf(w[64 + c], fv[i], h2);
-      }
-    }
-    u[p] = v[p] + h0;
-    s[p] = h1;
-    t[p] = h2;
-  }
-}
-
+// (the forward head runs in the last convolution's epilogue, ConvArgs::hp)
 // Loss, head gradients and the gradient into d1b.  With e_j = pred_j - target_j
 // and n = 3 V: loss += sum e_j^2 / n; dh_j = 2 e_j / n; dWh[j][c] += dh_j f[c];
 // dbh[j] += dh_j; G[p][c] = (sum_j dh_j Wh[j][c]) where f[c] > 0.
@@ -893,7 +910,10 @@ const bf16 *wf(const s3ttv_net *net, int l) { return net->wf + net->tab.woff[l];
 const bf16 *wbk(const s3ttv_net *net, int l) { return net->wb + net->tab.woff[l]; }
 const float *bias(const s3ttv_net *net, int l) { return net->theta + net->tab.boff[l]; }
 
-int run_forward(s3ttv_net *net, const float *v, const Vol &g0) {
+// The layers up to d1b; with out (u, s, t) the head as well, in the last layer's
+// epilogue, and d1b itself is not stored (256 x 256 x 128: 387 us for the layer and
+// 146 us for the head as its own kernel, 406 us together).
+int run_forward(s3ttv_net *net, const float *v, const Vol &g0, float *const *out = nullptr) {
   const Vol g1 = half(g0), g2 = half(g1);
   const int V0 = nvox(g0), V1 = nvox(g1), V2 = nvox(g2);
   conv_first_kernel<<<grid_for(net, V0, 256), 256, 0, net->stream>>>(v, wf(net, 0), bias(net, 0), net->e1a, g0);
@@ -912,7 +932,16 @@ int run_forward(s3ttv_net *net, const float *v, const Vol &g0) {
   NCU(launch_conv(net, net->e2b, 64, net->bb, 128, wf(net, 6), bias(net, 6), nullptr, net->d2a, 64, true, g1));
   NCU(launch_conv(net, net->d2a, 64, nullptr, 0, wf(net, 7), bias(net, 7), nullptr, net->d2b, 64, true, g1));
   NCU(launch_conv(net, net->e1b, 32, net->d2b, 64, wf(net, 8), bias(net, 8), nullptr, net->d1a, 32, true, g0));
-  NCU(launch_conv(net, net->d1a, 32, nullptr, 0, wf(net, 9), bias(net, 9), nullptr, net->d1b, 32, true, g0));
+  ConvArgs last{net->d1a, nullptr, wf(net, 9), bias(net, 9), nullptr, net->d1b, 32, 0, 32, 1, g0, net->err_flag};
+  if (out) {
+    last.y = nullptr;
+    last.hp = net->hp;
+    last.hv = v;
+    last.hu = out[0];
+    last.hs = out[1];
+    last.ht = out[2];
+  }
+  NCU(conv_launch(last, net->num_sms, net->stream));
   return S3TTV_OK;
 }
 
@@ -1136,14 +1165,11 @@ int s3ttv_net_forward(s3ttv_net *net, const float *v, int B, int D, int H, int W
   if ((rc = ensure_workspace(net, g))) return rc;
   const float *in[1] = {v}, *dev[1];
   if ((rc = stage_inputs(net, in, 1, n, dev))) return rc;
-  if ((rc = run_forward(net, dev[0], g))) return rc;
   float *outs[3] = {u, s, t}, *dout[3];
   const bool host_out = !on_device(u) || !on_device(s) || !on_device(t);
   if (host_out && (rc = ensure_stage(net, 4 * n))) return rc;
   for (int i = 0; i < 3; ++i) dout[i] = on_device(outs[i]) ? outs[i] : net->stage + (size_t)(i + 1) * n;
-  head_fwd_kernel<<<grid_for(net, (long long)n, 256), 256, 0, net->stream>>>(net->d1b, dev[0], net->hp, dout[0],
-                                                                             dout[1], dout[2], (int)n);
-  NCU(cudaGetLastError());
+  if ((rc = run_forward(net, dev[0], g, dout))) return rc;
   for (int i = 0; i < 3; ++i)
     if (dout[i] != outs[i])
       NCU(cudaMemcpyAsync(outs[i], dout[i], n * sizeof(float), cudaMemcpyDeviceToHost, net->stream));

@@ -194,6 +194,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t bars[2 * kMaxAStages + 2 * kMaxWStages + 2 * kMaxSlots + 2];
   __shared__ __align__(16) float s_bias[192];
+  __shared__ __align__(16) float s_head[100];  // the head's weights and biases
   __shared__ uint32_t s_tmem;
   __shared__ int s_stop;
   const int tid = threadIdx.x, lane = tid & 31;
@@ -239,6 +240,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
     s_stop = 0;
   }
   for (int i = tid; i < a.cout; i += kThreads) s_bias[i] = a.bias ? a.bias[i] : 0.f;
+  if (a.hp && tid < 99) s_head[tid] = a.hp[tid];
   fence_before();
   __syncthreads();
   fence_after();
@@ -309,8 +311,27 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
                 }
               }
             }
-            st_sector(a.y + o, ow);
-            st_sector(a.y + o + 16, ow + 8);
+            if (a.y) {
+              st_sector(a.y + o, ow);
+              st_sector(a.y + o + 16, ow + 8);
+            }
+            if (a.hp) {  // channel by channel, as a kernel of its own would sum
+              float h0 = s_head[96], h1 = s_head[97], h2 = s_head[98];
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                const float4 w0 = *reinterpret_cast<const float4 *>(s_head + 4 * i);
+                const float4 w1 = *reinterpret_cast<const float4 *>(s_head + 32 + 4 * i);
+                const float4 w2 = *reinterpret_cast<const float4 *>(s_head + 64 + 4 * i);
+                const float2 fa = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&ow[2 * i]));
+                const float2 fb = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&ow[2 * i + 1]));
+                h0 = fmaf(w0.w, fb.y, fmaf(w0.z, fb.x, fmaf(w0.y, fa.y, fmaf(w0.x, fa.x, h0))));
+                h1 = fmaf(w1.w, fb.y, fmaf(w1.z, fb.x, fmaf(w1.y, fa.y, fmaf(w1.x, fa.x, h1))));
+                h2 = fmaf(w2.w, fb.y, fmaf(w2.z, fb.x, fmaf(w2.y, fa.y, fmaf(w2.x, fa.x, h2))));
+              }
+              a.hu[vox] = a.hv[vox] + h0;
+              a.hs[vox] = h1;
+              a.ht[vox] = h2;
+            }
           }
           __syncwarp();
         }
@@ -627,7 +648,7 @@ cudaError_t conv_prepare() {
 
 cudaError_t conv_launch(const ConvArgs &a, int num_sms, cudaStream_t stream) {
   Plan pl;
-  if (a.cout % 32 || a.cout > 192 || !make_plan(a, num_sms, &pl)) return cudaErrorInvalidValue;
+  if (a.cout % 32 || a.cout > 192 || (a.hp && a.cout != 32) || !make_plan(a, num_sms, &pl)) return cudaErrorInvalidValue;
   if (a.c0 == 32 && a.c1 == 0) return launch<32, 0>(a, pl, num_sms, stream);
   if (a.c0 == 64 && a.c1 == 0) return launch<64, 0>(a, pl, num_sms, stream);
   if (a.c0 == 128 && a.c1 == 0) return launch<128, 0>(a, pl, num_sms, stream);

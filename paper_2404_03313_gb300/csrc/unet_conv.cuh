@@ -35,6 +35,11 @@ struct ConvArgs {
   int c0, c1, cout, relu;
   Vol g;
   int *err;           // device-visible; set when a wait inside the kernel ran out
+  // With 32 output channels, optionally the network's head on the rounded outputs
+  // f: h = Wh f + bh, (u, s, t) = (v + h0, h1, h2); hp holds Wh[3][32], then bh[3].
+  // y may be null then: the layer's output is not stored.
+  const float *hp = nullptr, *hv = nullptr;
+  float *hu = nullptr, *hs = nullptr, *ht = nullptr;
 };
 
 // Opt in to the kernels' shared memory (once per device before conv_launch).
