@@ -140,7 +140,7 @@ enum {
                                       context stays usable (host-side fault injection)    */
   S3TTV_OPT_NVTX = 15,             /* 1: NVTX ranges around each API call and each kernel
                                       class as a pass is enqueued (primal, l1-ball
-                                      thresholds, block dual, dual, finalize), for
+                                      thresholds, block dual, dual), for          
                                       profilers; 0 (default): none                        */
   S3TTV_OPT_JACOBI_POLISH_TOL = 16, /* relative orthogonality below which a pair of rows
                                       of the block eigen-solve is left as it is (0 <
@@ -234,10 +234,11 @@ enum { S3TTV_SPECTRAL_PERIODIC = 0, S3TTV_SPECTRAL_OPEN = 1 };
 /* Kernel classes reported by s3ttv_kernel_stats. */
 enum {
   S3TTV_KERNEL_PRIMAL = 0,     /* steps 2-7 for u, arguments of steps 3-4           */
-  S3TTV_KERNEL_L1_SEARCH = 1,  /* l1-ball thresholds of steps 3-4 (5 launches/pass) */
+  S3TTV_KERNEL_L1_SEARCH = 1,  /* l1-ball thresholds of steps 3-4 (levels 2 and 3: level
+                                  1 comes with the primal step) and D D_s ubar          */
   S3TTV_KERNEL_BLOCK_DUAL = 2, /* steps 8-11: block duals and their singular values */
-  S3TTV_KERNEL_DUAL = 3,       /* steps 3-4 finish, 12, 13                          */
-  S3TTV_KERNEL_FINALIZE = 4,   /* step 14 scalar and the stop rule                  */
+  S3TTV_KERNEL_DUAL = 3,       /* steps 3-4 finish, 12-14, the stop rule            */
+  S3TTV_KERNEL_FINALIZE = 4,   /* no launches: done by the dual step's last CTA     */
   S3TTV_KERNEL_CLASSES = 5
 };
 
@@ -273,8 +274,9 @@ int s3ttv_set_option(s3ttv_ctx *ctx, int key, double value);
 long long s3ttv_workspace_bytes(const s3ttv_ctx *ctx);
 
 /* Number of kernels the passes of Alg. 1 (s3ttv_iterate, s3ttv_solve,
- * s3ttv_solve_batched) have launched on this context since it was created (10
- * per pass of each problem, plus one per problem and call). */
+ * s3ttv_solve_batched) have launched on this context since it was created (5
+ * per pass of each problem, 6 with the FP64 re-solve, plus one per problem and
+ * call). */
 long long s3ttv_launch_count(const s3ttv_ctx *ctx);
 
 /* With S3TTV_OPT_PROFILE on: total device milliseconds (ms[c]) and launches

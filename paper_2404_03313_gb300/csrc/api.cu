@@ -86,7 +86,9 @@ namespace {
 
 constexpr int kMaxGrid = 4096;
 constexpr int kMaxK = kMaxLargeK;  // k <= 5: block_dual.cu; 6..16: block_dual_large.cu
-constexpr int kLaunchesPerPass = 10;  // kernels enqueue_pass launches (block-dual regularisers, no re-solve)
+// kernels enqueue_pass launches (without the re-solve): primal, l1 level 2 (with D D_s ubar
+// for the block-dual regularisers), l1 level 3, the regulariser's dual, dual
+constexpr int kLaunchesPerPass = 5;
 constexpr int kFbQueueMax = 1 << 16;  // entries of the FP64 re-solve queue
 
 int fail(s3ttv_ctx *c, int status, const char *fmt, ...) {
@@ -159,12 +161,13 @@ bool is_ssst(const s3ttv_ctx *c) { return c->reg == S3TTV_REG_SSST; }
 // parts of a block row: [D_v | D_h] (S3TTV, STV) or SSST's [D_v | D_h | D_s]
 int row_parts(const s3ttv_ctx *c) { return is_ssst(c) ? 3 : 2; }
 
+// CTAs of the elementwise kernels (512 threads, float4 pieces): at most two per SM.
 int elementwise_grid(const s3ttv_ctx *c, long long n) {
-  long long g = (n + 255) / 256;
-  long long cap = (long long)c->num_sms * 8;
+  long long g = (n + 2047) / 2048;
+  long long cap = (long long)c->num_sms * 2;
   if (cap > kMaxGrid) cap = kMaxGrid;
   if (g > cap) g = cap;
-  if (g < 1) g = 1;
+  if (g < 2) g = 2;
   return (int)g;
 }
 
@@ -626,7 +629,7 @@ BlockDualArgs make_bd_args(s3ttv_ctx *ctx, int par, const BdShape &bd) {
 
 // One pass of Alg. 1 (part 0), or its steps before the block duals (part 1:
 // primal step, l1-ball thresholds, D D_s ubar) or after them (part 2: the FP64
-// re-solve queue, the dual step, finalize); the batched solve launches the
+// re-solve queue, the dual step with the stop rule); the batched solve launches the
 // block duals of all its problems in between.
 int enqueue_pass(s3ttv_ctx *ctx, int par, int grid_e, const BdShape &bd,
                  cudaEvent_t *ev, int part = 0) {
@@ -648,8 +651,10 @@ int enqueue_pass(s3ttv_ctx *ctx, int par, int grid_e, const BdShape &bd,
   PrimalArgs pa;
   pa.Zv = ctx->Zv[par];
   pa.Zh = ctx->Zh[par];
-  pa.Znv = ctx->Zv[par ^ 1];
-  pa.Znh = ctx->Zh[par ^ 1];
+  // SSTV's and HSSTV's dual steps write Z, the block duals add into it
+  const bool blocks = ctx->reg != S3TTV_REG_SSTV && !is_hsstv(ctx);
+  pa.Znv = blocks ? ctx->Zv[par ^ 1] : nullptr;
+  pa.Znh = blocks ? ctx->Zh[par ^ 1] : nullptr;
   pa.u = ctx->u;
   pa.ubar = ctx->ubar;
   pa.s = ctx->s;
@@ -680,7 +685,7 @@ int enqueue_pass(s3ttv_ctx *ctx, int par, int grid_e, const BdShape &bd,
   }
   CU(launch_primal(pa, grid_e, st));
   if (ev) CU(cudaEventRecord(ev[1], st));
-  ph.next("l1-ball thresholds (steps 3-4)");
+  ph.next("l1-ball thresholds (steps 3-4), D D_s ubar");
 
   L1Args la;
   la.x[0] = ctx->zs;
@@ -690,11 +695,14 @@ int enqueue_pass(s3ttv_ctx *ctx, int par, int grid_e, const BdShape &bd,
   la.sc = ctx->sc;
   la.hcnt = ctx->hcnt;
   la.hsum = ctx->hsum;
-  CU(launch_l1_scan(la, 1, st));
-  CU(launch_l1_hist(la, 2, grid_e, st));
-  CU(launch_l1_scan(la, 2, st));
-  CU(launch_l1_hist(la, 3, grid_e, st));
-  CU(launch_l1_scan(la, 3, st));
+  // level 1 came with the primal step; level 2 comes with D D_s ubar where a block
+  // dual follows
+  if (blocks)
+    CU(launch_xfield(ctx->ubar, ctx->Fv, ctx->Fh, dm, grid_e, st, ctx->open_s,
+                     ctx->reg == S3TTV_REG_STV || is_ssst(ctx), ctx->Fs, &la));
+  else
+    CU(launch_l1_level(la, 2, grid_e, st));
+  CU(launch_l1_level(la, 3, grid_e, st));
   if (ev) CU(cudaEventRecord(ev[2], st));
 
   ph.next("block dual (steps 8-11)");
@@ -705,10 +713,8 @@ int enqueue_pass(s3ttv_ctx *ctx, int par, int grid_e, const BdShape &bd,
     CU(launch_hsstv_dual(ctx->ubar, ctx->Y, ctx->Zv[par ^ 1], ctx->Zh[par ^ 1], dm, (float)ctx->gam[3],
                          ctx->hsstv_omega, ctx->reg == S3TTV_REG_HSSTV2, grid_e, st));
   } else {
-  CU(launch_xfield(ctx->ubar, ctx->Fv, ctx->Fh, dm, grid_e, st, ctx->open_s,
-                   ctx->reg == S3TTV_REG_STV || is_ssst(ctx), ctx->Fs));
   if (part == 1) {
-    ctx->launches += 7;  // primal, three scans, two histograms, xfield
+    ctx->launches += 3;  // primal, xfield with the second level, third level
     return S3TTV_OK;
   }
   const BlockDualArgs ba = make_bd_args(ctx, par, bd);
@@ -727,7 +733,7 @@ int enqueue_pass(s3ttv_ctx *ctx, int par, int grid_e, const BdShape &bd,
   if (ev) CU(cudaEventRecord(ev[3], st));
   }  // part != 2
 
-  ph.next("dual (steps 12-13)");
+  ph.next("dual (steps 12-14, stop rule)");
   DualArgs da;
   da.zs = ctx->zs;
   da.zt = ctx->zt;
@@ -744,26 +750,20 @@ int enqueue_pass(s3ttv_ctx *ctx, int par, int grid_e, const BdShape &bd,
   da.g3 = (float)ctx->gam[5];
   da.sc = ctx->sc;
   da.part = ctx->part + 2 * grid_e;
+  da.part_primal = ctx->part;
+  da.grid_p = grid_e;
+  da.eps = ctx->eps;
+  da.g3d = ctx->gam[5];
   CU(launch_dual(da, grid_e, st));
-  if (ev) CU(cudaEventRecord(ev[4], st));
-
-  FinalizeArgs fa;
-  fa.sc = ctx->sc;
-  fa.part_primal = ctx->part;
-  fa.grid_p = grid_e;
-  fa.part_dual = ctx->part + 2 * grid_e;
-  fa.grid_d = grid_e;
-  fa.eps = ctx->eps;
-  fa.g3 = ctx->gam[5];
-  ph.next("finalize (step 14, stop rule)");
-  CU(launch_finalize(fa, st));
-  if (ev) CU(cudaEventRecord(ev[5], st));
+  if (ev) {
+    CU(cudaEventRecord(ev[4], st));
+    CU(cudaEventRecord(ev[5], st));
+  }
   if (part == 2) {
-    ctx->launches += 2;  // dual, finalize (the block duals are counted by the batch)
+    ctx->launches += 1;  // dual (the block duals are counted by the batch)
     return S3TTV_OK;
   }
-  // SSTV and HSSTV: one elementwise dual kernel in place of xfield + block dual
-  ctx->launches += (ctx->reg == S3TTV_REG_SSTV || is_hsstv(ctx)) ? kLaunchesPerPass - 1 : kLaunchesPerPass;
+  ctx->launches += kLaunchesPerPass;
   return S3TTV_OK;
 }
 
@@ -806,7 +806,7 @@ int collect_events(s3ttv_ctx *ctx, int passes) {
       float ms = 0.f;
       CU(cudaEventElapsedTime(&ms, e[c], e[c + 1]));
       ctx->prof_ms[c] += ms;
-      ctx->prof_n[c] += c == S3TTV_KERNEL_L1_SEARCH ? 5 : 1;
+      ctx->prof_n[c] += c == S3TTV_KERNEL_L1_SEARCH ? 2 : c == S3TTV_KERNEL_FINALIZE ? 0 : 1;
     }
   }
   return S3TTV_OK;
@@ -1029,6 +1029,7 @@ int s3ttv_setup(s3ttv_ctx *ctx, const float *v, int N1, int N2, int N3, float ep
   BdShape bd;
   if ((rc = block_dual_shape(ctx, dm, k, &bd))) return rc;
   if ((rc = ensure_problem_buffers(ctx, dm, k))) return rc;
+  CU(primal_prepare());
   ctx->dm = dm;
   ctx->k = k;
   ctx->eps = eps;
@@ -1614,8 +1615,7 @@ int s3ttv_l1_ball(s3ttv_ctx *ctx, const float *x, float *out, long long n, doubl
   la.hsum = ctx->hsum;
   const int grid = elementwise_grid(ctx, n);
   for (int level = 1; level <= 3; ++level) {
-    CU(launch_l1_hist(la, level, grid, ctx->stream));
-    CU(launch_l1_scan(la, level, ctx->stream));
+    CU(launch_l1_level(la, level, grid, ctx->stream));
   }
   CU(launch_soft_threshold(xin, xout, n, ctx->sc, 0, ctx->stream));
   if (!od) CU(cudaMemcpyAsync(out, xout, sizeof(float) * n, cudaMemcpyDeviceToHost, ctx->stream));

@@ -993,6 +993,7 @@ __device__ __forceinline__ void prefetch_rows(const float *Yl, int N3p) {
 // instead of FP32 CUDA cores.
 template <int K, int MINB, bool TC>
 __global__ void __launch_bounds__(kNW * 32, MINB) block_dual_kernel(BlockDualArgs a) {
+  chained();
   using S = Shape<K>;
   constexpr int n = S::n, GS = S::GS, TR = S::TR, NT = S::NT, TS = S::TS, RH = S::RH, MH = S::MH,
                 MS = S::MS;
@@ -1621,6 +1622,7 @@ __device__ void stream_block(const BlockDualArgs &a, long long l, float *bufs, u
 
 template <int K>
 __global__ void __launch_bounds__(kSW * 32, 4) block_dual_stream_kernel(BlockDualArgs a) {
+  chained();
   extern __shared__ __align__(16) float smem[];
   if (a.sc->done) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1643,6 +1645,7 @@ __global__ void __launch_bounds__(kSW * 32, 4) block_dual_stream_kernel(BlockDua
 template <int K>
 __global__ void __launch_bounds__(kSW * 32, 4) block_dual_stream_batch_kernel(const BatchDual *items, int n,
                                                                               long long total) {
+  chained();
   extern __shared__ __align__(16) float smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float *bufs = smem + warp * StreamLayout<K>::per_warp;
@@ -1810,15 +1813,13 @@ cudaError_t block_dual_batch_prepare(int k, int *ctas_per_sm) {
 cudaError_t launch_block_dual_batch(int k, const BatchDual *items, int n, long long total, int grid, cudaStream_t st) {
   BatchFn f = batch_kernel(k);
   if (!f) return cudaErrorInvalidValue;
-  f<<<grid, kSW * 32, batch_smem(k), st>>>(items, n, total);
-  return cudaGetLastError();
+  return launch_chained(f, grid, kSW * 32, batch_smem(k), st, items, n, total);
 }
 
 cudaError_t launch_block_dual(const BlockDualArgs &a, const BdVariant &v, int grid, size_t smem, cudaStream_t st) {
   KernelFn f = kernel_for(v);
   if (!f) return cudaErrorInvalidValue;
-  f<<<grid, kNW * 32, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_chained(f, grid, kNW * 32, smem, st, a);
 }
 
 }  // namespace s3ttv

@@ -260,6 +260,7 @@ template <int K, bool ST, int PARTS>
 __global__ void __launch_bounds__(large_warps<K, ST, PARTS>() * 32,
                                   large_warps<K, ST, PARTS>() == 4 ? 4 : (large_warps<K, ST, PARTS>() == 16 ? 1 : 2))
     block_dual_large_kernel(BlockDualArgs a) {
+  chained();
   constexpr int LW = large_warps<K, ST, PARTS>(), LT = LW * 32;
   constexpr int k = K;
   constexpr int NR = ST ? 2 * K * K : K * K;            // rows of a block matrix
@@ -1062,8 +1063,7 @@ cudaError_t launch_block_dual_large(const BlockDualArgs &a, int k, bool stacked,
   if (!f) return cudaErrorInvalidValue;
   const size_t rows = block_dual_large_rows_floats(k, stacked, parts);
   if (rows && (!a.rows || rows * (size_t)grid > a.rows_cap)) return cudaErrorInvalidValue;
-  f<<<grid, block_dual_large_threads(k, stacked, parts), smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_chained(f, grid, block_dual_large_threads(k, stacked, parts), smem, st, a);
 }
 
 }  // namespace s3ttv

@@ -3,40 +3,27 @@
 // scalar finish of step 14 and the stop rule (eq. StopCri_simulated), and the
 // layout helpers.  All are HBM-bound streams over [N1][N2][N3p] cubes.
 #include <math.h>
-#include "s3ttv_internal.cuh"
+#include "l1_select.cuh"
 
 namespace s3ttv {
 namespace {
 
-// Block-wide sum of two doubles (blockDim.x a multiple of 32, <= 1024).
+// The CTA's FP64 sums of NV floats per thread, value v by warp v (result in its lane
+// 0).  One warp per value adds kSelThreads / 32 floats per lane: FP64 runs at two
+// operations a cycle and SM, so a shuffle tree in every warp took 1.3 us.
 template <int NV>
-__device__ void block_sum(double (&v)[NV], double (*red)[32]) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+__device__ double block_sum(const float (&v)[NV], float (*red)[kSelThreads]) {
 #pragma unroll
-  for (int k = 0; k < NV; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(kFull, v[k], o);
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < NV; ++k) red[k][w] = v[k];
+  for (int k = 0; k < NV; ++k) red[k][threadIdx.x] = v[k];
   __syncthreads();
-  if (w == 0) {
-    const int nw = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double s = 0.0;
+  if (w < NV) {
+    for (int i = lane; i < kSelThreads; i += 32) s += (double)red[w][i];
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      v[k] = lane < nw ? red[k][lane] : 0.0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(kFull, v[k], o);
-    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(kFull, s, o);
   }
-}
-
-__device__ __forceinline__ void hist_add(unsigned *cnt, float *sum, float z) {
-  const unsigned bits = __float_as_uint(z) & 0x7fffffffu;
-  if (bits == 0u) return;  // zeros never enter the active set
-  const unsigned key = bits >> 20;
-  atomicAdd(&cnt[key], 1u);
-  atomicAdd(&sum[key], __uint_as_float(bits));
+  return s;
 }
 
 // Work unit of primal_kernel and dual_kernel: one float4 chunk (4 consecutive
@@ -52,22 +39,21 @@ __device__ __forceinline__ float comp(const float4 &v, int e) { return e == 0 ? 
 //   ubar = 2 u+ - u                                                  (step 5)
 //   zs   = s - gs y3,   zt = t - gt (D_v^T y2 + y3)                 (steps 3, 4)
 // with y3 = c3 d and Z = sum_l P_l^T Y_l.  Also: sum (u+ - u)^2 and sum u^2 for
-// the stop rule, the first radix level of |zs| and |zt|, and zeroing of the next
+// the stop rule, the first radix level of |zs| and |zt| (histograms by every CTA,
+// the thresholds narrowed by the one that finishes last), and zeroing of the next
 // Z accumulator.  EXTRA: 0 S3TTV, STV, SSTV; 1 HSSTV (+ omega D^T of the
 // first-order dual pair); 2 SSST (+ D_s^T Zs, and Zns zeroed).
 template <int EXTRA>
-__global__ void __launch_bounds__(256) primal_kernel(PrimalArgs a) {
-  __shared__ unsigned s_cnt[2 * kHistBins];
-  __shared__ float s_sum[2 * kHistBins];
-  __shared__ double s_red[2][32];
+__global__ void __launch_bounds__(kSelThreads, 2) primal_kernel(PrimalArgs a) {
+  chained();
+  extern __shared__ __align__(16) BinSums s_hist[];  // of zs and of zt
+  __shared__ float s_red[2][kSelThreads];
   if (a.sc->done) return;
   // this pass's FP64 re-solve queue starts empty (the block dual runs after this
   // kernel, the previous pass's re-solve before it)
   if (blockIdx.x == 0 && threadIdx.x == 0) a.sc->fb_count = 0u;
-  for (int i = threadIdx.x; i < 2 * kHistBins; i += blockDim.x) {
-    s_cnt[i] = 0u;
-    s_sum[i] = 0.f;
-  }
+  for (int i = threadIdx.x; i < (int)(2 * sizeof(BinSums) / 16); i += blockDim.x)
+    reinterpret_cast<uint4 *>(s_hist)[i] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
   const Dims dm = a.dm;
   const int N3p = dm.N3p, C4 = N3p >> 2, N2 = dm.N2;
@@ -81,8 +67,10 @@ __global__ void __launch_bounds__(256) primal_kernel(PrimalArgs a) {
     const size_t p0 = (size_t)pix * N3p + b0;
     const size_t pim = ((size_t)(i == 0 ? dm.N1 - 1 : i - 1) * N2 + j) * N3p + b0;
     const size_t pjm = ((size_t)i * N2 + (j == 0 ? N2 - 1 : j - 1)) * N3p + b0;
-    st4(a.Znv + p0, zero4);
-    st4(a.Znh + p0, zero4);
+    if (a.Znv) {
+      st4(a.Znv + p0, zero4);
+      st4(a.Znh + p0, zero4);
+    }
     if (EXTRA == 2) st4(a.Zns + p0, zero4);
     // w = D_v^T Zv + D_h^T Zh at bands b0..b0+3 and at the band before b0
     // (periodic over the N3 true bands)
@@ -121,8 +109,8 @@ __global__ void __launch_bounds__(256) primal_kernel(PrimalArgs a) {
         const float dl = v - u;
         du2 = fmaf(dl, dl, du2);
         u2 = fmaf(u, u, u2);
-        hist_add(s_cnt, s_sum, zs[e]);
-        hist_add(s_cnt + kHistBins, s_sum + kHistBins, zt[e]);
+        hist_add<1>(s_hist[0], 0u, zs[e]);
+        hist_add<1>(s_hist[1], 0u, zt[e]);
       } else {  // padding bands stay 0
         un[e] = comp(u4, e);
         ub[e] = zs[e] = zt[e] = 0.f;
@@ -133,18 +121,54 @@ __global__ void __launch_bounds__(256) primal_kernel(PrimalArgs a) {
     st4(a.zs + p0, make_float4(zs[0], zs[1], zs[2], zs[3]));
     st4(a.zt + p0, make_float4(zt[0], zt[1], zt[2], zt[3]));
   }
-  double v[2] = {(double)du2, (double)u2};
-  block_sum<2>(v, s_red);
-  if (threadIdx.x == 0) {
-    a.part[blockIdx.x] = v[0];
-    a.part[gridDim.x + blockIdx.x] = v[1];
-  }
-  __syncthreads();
+  const float v[2] = {du2, u2};
+  const double sum = block_sum<2>(v, s_red);
+  if ((threadIdx.x & 31) == 0 && threadIdx.x < 64) a.part[(threadIdx.x >> 5) * gridDim.x + blockIdx.x] = sum;
   for (int i = threadIdx.x; i < 2 * kHistBins; i += blockDim.x) {
-    const unsigned c = s_cnt[i];
+    const BinSums &h = s_hist[i / kHistBins];
+    const unsigned c = h.cnt[i % kHistBins];
     if (c) {
       atomicAdd(&a.hcnt[i], c);
-      atomicAdd(&a.hsum[i], (double)s_sum[i]);
+      atomicAdd(&a.hsum[i], bin_sum<1>(h, 0u, i % kHistBins));
+    }
+  }
+  if (last_cta(&a.sc->ticket[2], gridDim.x)) {
+    const int pb = threadIdx.x / kTeam;  // a team per threshold
+    if (pb < 2) l1_scan<kHistBins / kTeam>(a.sc, a.hcnt + pb * kHistBins, a.hsum + pb * kHistBins, pb, 1, pb);
+  }
+}
+
+// Step 14 and the stop rule, by the CTA of dual_kernel that finishes last.
+__device__ void finalize(const DualArgs &a, int grid_d) {
+  __shared__ double s_sum[3];
+  Scalars *sc = a.sc;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (w < 3) {  // a warp per sum
+    const double *p = w < 2 ? a.part_primal + w * a.grid_p : a.part;
+    const int n = w < 2 ? a.grid_p : grid_d;
+    double s = 0.0;
+    for (int i = lane; i < n; i += 32) s += __ldcg(p + i);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(kFull, s, o);
+    if (lane == 0) s_sum[w] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const double du2 = s_sum[0], u2 = s_sum[1], d2 = s_sum[2];
+    const double nd = sqrt(d2);
+    sc->c3 = nd > a.eps ? a.g3d * (1.0 - a.eps / nd) : 0.0;
+    const double rel = u2 > 0.0 ? sqrt(du2) / sqrt(u2) : sqrt(du2);
+    sc->rel = rel;
+    sc->iter += 1;
+    if (!isfinite(rel) || !isfinite(d2)) {
+      sc->status = -4;
+      sc->done = 1;
+    } else if (rel < (double)sc->tol) {
+      sc->status = 1;
+      sc->done = 1;
+    } else if (sc->iter >= sc->iter_limit) {
+      sc->status = 2;
+      sc->done = 1;
     }
   }
 }
@@ -153,9 +177,10 @@ __global__ void __launch_bounds__(256) primal_kernel(PrimalArgs a) {
 //   s+ = S_tau_s(zs), t+ = S_tau_t(zt), sbar = 2 s+ - s, tbar = 2 t+ - t
 //   y2 += g2 D_v tbar                                                (step 12)
 //   y3' = y3 + g3 (ubar + sbar + tbar),  d = y3' / g3 - v            (step 13)
-// (step 14 scales d by the scalar c3 of finalize_kernel), and sum d^2.
-__global__ void __launch_bounds__(256) dual_kernel(DualArgs a) {
-  __shared__ double s_red[1][32];
+// (step 14 scales d by the scalar c3 of finalize()), and sum d^2.
+__global__ void __launch_bounds__(kSelThreads, 2) dual_kernel(DualArgs a) {
+  chained();
+  __shared__ float s_red[1][kSelThreads];
   if (a.sc->done) return;
   const Dims dm = a.dm;
   const int N3p = dm.N3p, C4 = N3p >> 2, N2 = dm.N2;
@@ -197,40 +222,10 @@ __global__ void __launch_bounds__(256) dual_kernel(DualArgs a) {
     st4(a.y2 + p0, make_float4(y2n[0], y2n[1], y2n[2], y2n[3]));
     st4(a.d + p0, make_float4(dn[0], dn[1], dn[2], dn[3]));
   }
-  double v[1] = {(double)d2};
-  block_sum<1>(v, s_red);
-  if (threadIdx.x == 0) a.part[blockIdx.x] = v[0];
-}
-
-__global__ void __launch_bounds__(256) finalize_kernel(FinalizeArgs a) {
-  __shared__ double s_red[3][32];
-  Scalars *sc = a.sc;
-  if (sc->done) return;
-  double v[3] = {0.0, 0.0, 0.0};
-  for (int i = threadIdx.x; i < a.grid_p; i += blockDim.x) {
-    v[0] += a.part_primal[i];
-    v[1] += a.part_primal[a.grid_p + i];
-  }
-  for (int i = threadIdx.x; i < a.grid_d; i += blockDim.x) v[2] += a.part_dual[i];
-  block_sum<3>(v, s_red);
-  if (threadIdx.x == 0) {
-    const double du2 = v[0], u2 = v[1], d2 = v[2];
-    const double nd = sqrt(d2);
-    sc->c3 = nd > a.eps ? a.g3 * (1.0 - a.eps / nd) : 0.0;
-    const double rel = u2 > 0.0 ? sqrt(du2) / sqrt(u2) : sqrt(du2);
-    sc->rel = rel;
-    sc->iter += 1;
-    if (!isfinite(rel) || !isfinite(d2)) {
-      sc->status = -4;
-      sc->done = 1;
-    } else if (rel < (double)sc->tol) {
-      sc->status = 1;
-      sc->done = 1;
-    } else if (sc->iter >= sc->iter_limit) {
-      sc->status = 2;
-      sc->done = 1;
-    }
-  }
+  const float v[1] = {d2};
+  const double sum = block_sum<1>(v, s_red);
+  if (threadIdx.x == 0) a.part[blockIdx.x] = sum;
+  if (last_cta(&a.sc->ticket[3], gridDim.x)) finalize(a, gridDim.x);
 }
 
 __global__ void pad_cube_kernel(const float *__restrict__ src, float *__restrict__ dst, Dims dm, float scale) {
@@ -271,15 +266,24 @@ __global__ void Y_to_internal_kernel(const float *__restrict__ ext, float *__res
   }
 }
 
-__global__ void Y_to_external_kernel(const float *__restrict__ in, float *__restrict__ ext, Dims dm, int n,
-                                     int stacked, int parts) {
-  const long long total = dm.P * n * parts * dm.N3;
-  const long long stride = (long long)gridDim.x * blockDim.x;
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += stride) {
-    const long long row = idx / (parts * dm.N3);
-    const int col = (int)(idx - row * parts * dm.N3);
-    const int b = stacked ? col % dm.N3 : col / parts, o = stacked ? col / dm.N3 : col % parts;
-    ext[idx] = in[row * parts * dm.N3p + (long long)o * dm.N3p + b];
+// A warp per block row, a lane per band: the part(s) of a row are read and written
+// in order, the paper layout's pairs (v_b, h_b) as 8-byte stores where ext allows
+// (pairs: 1).  An element per thread with its divisions took 2.59 ms at 304 x 304 x
+// 191, k = 5, this 1.2 ms.
+__global__ void __launch_bounds__(256) Y_to_external_kernel(const float *__restrict__ in, float *__restrict__ ext, Dims dm,
+                                                            int n, int stacked, int parts, int pairs) {
+  const int lane = threadIdx.x & 31, N3 = dm.N3, N3p = dm.N3p;
+  const long long rows = dm.P * n, stride = (long long)gridDim.x * 8;
+  for (long long row = blockIdx.x * 8LL + (threadIdx.x >> 5); row < rows; row += stride) {
+    const float *src = in + row * parts * N3p;
+    float *dst = ext + row * parts * N3;
+    if (pairs) {
+#pragma unroll 4
+      for (int b = lane; b < N3; b += 32) reinterpret_cast<float2 *>(dst)[b] = make_float2(src[b], src[N3p + b]);
+    } else {
+      for (int o = 0; o < parts; ++o)
+        for (int b = lane; b < N3; b += 32) dst[stacked ? o * N3 + b : parts * b + o] = src[o * N3p + b];
+    }
   }
 }
 
@@ -313,11 +317,27 @@ __global__ void Z_from_Y_kernel(const float *__restrict__ Y, float *__restrict__
 
 // Fv = D_v D_s ubar and Fh = D_h D_s ubar: the second-order differences the
 // structure tensors of eq. (SSST) are cut from, formed once per pass.
-__global__ void xfield_kernel(const float *__restrict__ ubar, float *__restrict__ Fv, float *__restrict__ Fh,
-                              Dims dm, int open_s, int first_order, float *__restrict__ Fs) {
+// The first 2 nh CTAs take the second level of the l1-ball thresholds of s and t
+// instead (independent of F): one launch for both.
+__global__ void __launch_bounds__(kSelThreads, 3) xfield_kernel(const float *__restrict__ ubar, float *__restrict__ Fv,
+                                                                float *__restrict__ Fh, Dims dm, int open_s,
+                                                                int first_order, float *__restrict__ Fs, L1Args l1,
+                                                                int nh) {
+  chained();
+  if ((int)blockIdx.x < 2 * nh) {
+    __shared__ BinSums s_hist;
+    const int pb = (int)blockIdx.x >= nh, cta = blockIdx.x - pb * nh;
+    if (l1.sc->done) return;
+    const L1State st = l1.sc->l1[pb];
+    if (st.mode != 0) return;  // decided at the first level
+    l1_hist<2, true>(l1, st, pb, (long long)cta * kSelThreads + threadIdx.x, (long long)nh * kSelThreads, s_hist);
+    if (last_cta(&l1.sc->ticket[pb], nh)) l1_scan_level<2>(l1, pb);
+    return;
+  }
+  const int first = (blockIdx.x - 2 * nh) * blockDim.x + threadIdx.x, stride = (gridDim.x - 2 * nh) * blockDim.x;
   const int N3p = dm.N3p, C4 = N3p >> 2, N2 = dm.N2;
   const int nch = (int)(dm.P * C4);
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nch; c += gridDim.x * blockDim.x) {
+  for (int c = first; c < nch; c += stride) {
     const int pix = (unsigned)c / (unsigned)C4, q = c - pix * C4, b0 = q << 2;
     const int i = (unsigned)pix / (unsigned)N2, j = pix - i * N2;
     const size_t p0 = (size_t)pix * N3p;
@@ -368,21 +388,21 @@ int grid_for(long long n) {
 
 }  // namespace
 
+cudaError_t primal_prepare() {
+  for (const auto kernel : {primal_kernel<0>, primal_kernel<1>, primal_kernel<2>}) {
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * sizeof(BinSums));
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 cudaError_t launch_primal(const PrimalArgs &a, int grid, cudaStream_t st) {
-  if (a.Zs) primal_kernel<2><<<grid, 256, 0, st>>>(a);
-  else if (a.Z1v) primal_kernel<1><<<grid, 256, 0, st>>>(a);
-  else primal_kernel<0><<<grid, 256, 0, st>>>(a);
-  return cudaGetLastError();
+  const auto kernel = a.Zs ? primal_kernel<2> : a.Z1v ? primal_kernel<1> : primal_kernel<0>;
+  return launch_chained(kernel, grid, kSelThreads, 2 * sizeof(BinSums), st, a);
 }
 
 cudaError_t launch_dual(const DualArgs &a, int grid, cudaStream_t st) {
-  dual_kernel<<<grid, 256, 0, st>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t st) {
-  finalize_kernel<<<1, 256, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_chained(dual_kernel, grid, kSelThreads, 0, st, a);
 }
 
 // SSTV's dual step (the l1 norm of D D_s u in place of the block nuclear
@@ -392,6 +412,7 @@ cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t st) {
 // Z = sum_l P_l^T Y_l becomes Y itself: written to (Zv, Zh).
 __global__ void sstv_dual_kernel(const float *__restrict__ ubar, float *__restrict__ Yv, float *__restrict__ Yh,
                                  float *__restrict__ Zv, float *__restrict__ Zh, Dims dm, float gY) {
+  chained();
   const int N3p = dm.N3p, C4 = N3p >> 2, N2 = dm.N2;
   const int nch = (int)(dm.P * C4);
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nch; c += gridDim.x * blockDim.x) {
@@ -433,6 +454,7 @@ __global__ void sstv_dual_kernel(const float *__restrict__ ubar, float *__restri
 // Y holds four internal cubes; the second-order pair is also written to Z.
 __global__ void hsstv_dual_kernel(const float *__restrict__ ubar, float *__restrict__ Y, float *__restrict__ Zv,
                                   float *__restrict__ Zh, Dims dm, float gY, float omega, int l12) {
+  chained();
   const int N3p = dm.N3p, C4 = N3p >> 2, N2 = dm.N2;
   const int nch = (int)(dm.P * C4);
   const size_t Np = (size_t)dm.Np;
@@ -480,14 +502,12 @@ __global__ void hsstv_dual_kernel(const float *__restrict__ ubar, float *__restr
 
 cudaError_t launch_hsstv_dual(const float *ubar, float *Y, float *Zv, float *Zh, Dims dm, float gY, float omega,
                               int l12, int grid, cudaStream_t st) {
-  hsstv_dual_kernel<<<grid, 256, 0, st>>>(ubar, Y, Zv, Zh, dm, gY, omega, l12);
-  return cudaGetLastError();
+  return launch_chained(hsstv_dual_kernel, 4 * grid, 256, 0, st, ubar, Y, Zv, Zh, dm, gY, omega, l12);
 }
 
 cudaError_t launch_sstv_dual(const float *ubar, float *Yv, float *Yh, float *Zv, float *Zh, Dims dm, float gY,
                              int grid, cudaStream_t st) {
-  sstv_dual_kernel<<<grid, 256, 0, st>>>(ubar, Yv, Yh, Zv, Zh, dm, gY);
-  return cudaGetLastError();
+  return launch_chained(sstv_dual_kernel, 4 * grid, 256, 0, st, ubar, Yv, Yh, Zv, Zh, dm, gY);
 }
 
 cudaError_t launch_pad_cube(const float *src, float *dst, Dims dm, float scale, cudaStream_t st) {
@@ -508,14 +528,18 @@ cudaError_t launch_Y_to_internal(const float *ext, float *in, Dims dm, int k, cu
 
 cudaError_t launch_Y_to_external(const float *in, float *ext, Dims dm, int k, cudaStream_t st, int stacked,
                                  int parts) {
-  Y_to_external_kernel<<<grid_for(dm.P * k * k * parts * dm.N3), 256, 0, st>>>(in, ext, dm, k * k, stacked, parts);
+  const long long rows = dm.P * k * k;
+  const int pairs = !stacked && parts == 2 && (reinterpret_cast<uintptr_t>(ext) & 7) == 0;
+  Y_to_external_kernel<<<(int)(rows < 8 * 4096 ? (rows + 7) / 8 : 4096), 256, 0, st>>>(in, ext, dm, k * k, stacked, parts,
+                                                                                   pairs);
   return cudaGetLastError();
 }
 
 cudaError_t launch_xfield(const float *ubar, float *Fv, float *Fh, Dims dm, int grid, cudaStream_t st, int open_s,
-                          int first_order, float *Fs) {
-  xfield_kernel<<<grid, 256, 0, st>>>(ubar, Fv, Fh, dm, open_s, first_order, Fs);
-  return cudaGetLastError();
+                          int first_order, float *Fs, const L1Args *l1) {
+  const int nh = l1 ? grid / 2 : 0;  // (grid: two CTAs per SM)
+  return launch_chained(xfield_kernel, grid + 2 * nh, kSelThreads, 0, st, ubar, Fv, Fh, dm, open_s, first_order, Fs,
+                        l1 ? *l1 : L1Args(), nh);
 }
 
 cudaError_t launch_Z_from_Y(const float *Y, float *Zv, float *Zh, Dims dm, int k, cudaStream_t st, float *Zs) {

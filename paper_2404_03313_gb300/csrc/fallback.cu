@@ -53,6 +53,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // k, stacked (rows 2r, 2r + 1: D_v, D_h parts of window pixel r) and parts
 // (paper layout: 2, or SSST's 3 parts of N3p bands per row) as in the FP32 kernels
 __global__ void __launch_bounds__(kFbThreads) fallback_kernel(BlockDualArgs a, int k, int stacked, int parts) {
+  chained();
   extern __shared__ __align__(16) double fsm[];
   if (a.sc->done) return;
   const unsigned queued = a.sc->fb_count;
@@ -228,8 +229,7 @@ cudaError_t fallback_prepare(size_t smem) {
 
 cudaError_t launch_fallback(const BlockDualArgs &a, int k, int stacked, int parts, int grid, size_t smem,
                             cudaStream_t st) {
-  fallback_kernel<<<grid, kFbThreads, smem, st>>>(a, k, stacked, parts);
-  return cudaGetLastError();
+  return launch_chained(fallback_kernel, grid, kFbThreads, smem, st, a, k, stacked, parts);
 }
 
 }  // namespace s3ttv

@@ -15,6 +15,30 @@
 
 namespace s3ttv {
 
+// The kernels of a pass are launched as programmatic dependents of one another:
+// chained() is the first statement of each, lets the next kernel's CTAs come in as
+// soon as this one's have all started, and waits for the kernel before to be done
+// (with its writes), so launch latency and CTA set-up overlap the tail of the
+// kernel before.  No kernel touches memory ahead of it.
+__device__ __forceinline__ void chained() {
+  asm volatile("griddepcontrol.launch_dependents;\n griddepcontrol.wait;\n" ::: "memory");
+}
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                                  A... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 constexpr int kHistBins = 2048;  // bins of the widest radix level
 constexpr unsigned kFull = 0xffffffffu;
 
@@ -50,6 +74,7 @@ struct Scalars {
   unsigned fb_count;  // blocks queued for the FP64 re-solve in this pass (reset by the primal step)
   unsigned fb_total;  // blocks re-solved in FP64 since the last s3ttv_iterate began
   unsigned long long fo_blocks;  // blocks whose clip came from the first-order update (statistics)
+  unsigned ticket[4];  // CTAs done: histograms of s and t, primal step, dual step (zero between kernels)
 };
 
 // Radix levels over the 31 magnitude bits of a float.
@@ -69,7 +94,7 @@ __device__ __forceinline__ float soft_threshold(float z, float tau, float tau_lo
 // ---- launch wrappers (each returns the launch error) ----
 struct PrimalArgs {
   const float *Zv, *Zh;   // sum_l P_l^T Y_l of the current Y
-  float *Znv, *Znh;       // next accumulation target, zeroed here
+  float *Znv, *Znh;       // next accumulation target, zeroed here (null: it is overwritten)
   float *u, *ubar;        // u is updated in place, ubar = 2u+ - u
   const float *s, *t, *y2, *d;
   float *zs, *zt;         // pre-projection arguments of steps 3 and 4
@@ -85,6 +110,7 @@ struct PrimalArgs {
   const float *Zs = nullptr;  // SSST: the spectral part, adds D_s^T Zs
   float *Zns = nullptr;       // its next accumulation target, zeroed here
 };
+cudaError_t primal_prepare();  // opt in to its shared memory, once per device before launch_primal
 cudaError_t launch_primal(const PrimalArgs &a, int grid, cudaStream_t st);
 
 struct DualArgs {
@@ -94,22 +120,14 @@ struct DualArgs {
   float g2, g3;
   Scalars *sc;
   double *part;           // [grid]: sum d^2
+  const double *part_primal;  // [2][grid_p], of the primal step
+  int grid_p;
+  double eps, g3d;        // step 14 (in FP64), run with the stop rule by the CTA that finishes last
 };
 cudaError_t launch_dual(const DualArgs &a, int grid, cudaStream_t st);
 
-struct FinalizeArgs {
-  Scalars *sc;
-  const double *part_primal;  // [2][grid_p]
-  int grid_p;
-  const double *part_dual;    // [grid_d]
-  int grid_d;
-  double eps;
-  double g3;
-};
-cudaError_t launch_finalize(const FinalizeArgs &a, cudaStream_t st);
-
-// l1-ball radix selection: histogram pass over up to two vectors and the scan
-// that narrows the threshold one level.
+// l1-ball radix selection: a level is the histogram of up to two vectors and the
+// narrowing of their thresholds.
 struct L1Args {
   const float *x[2];
   long long n;            // elements of each vector (both the same length)
@@ -118,8 +136,7 @@ struct L1Args {
   unsigned *hcnt;         // [2][kHistBins]
   double *hsum;           // [2][kHistBins]
 };
-cudaError_t launch_l1_hist(const L1Args &a, int level, int grid, cudaStream_t st);
-cudaError_t launch_l1_scan(const L1Args &a, int level, cudaStream_t st);
+cudaError_t launch_l1_level(const L1Args &a, int level, int grid, cudaStream_t st);
 cudaError_t launch_soft_threshold(const float *x, float *out, long long n, const Scalars *sc,
                                   int prob, cudaStream_t st);
 
@@ -218,8 +235,9 @@ cudaError_t launch_Y_to_external(const float *in, float *ext, Dims dm, int k, cu
 // open_s: the spectral difference stops at the last band (F's last band is 0)
 // first_order: F = (D_v u, D_h u) (STV) instead of the second-order differences;
 // with Fs as well, SSST's first-order parts (D_v u, D_h u, D_s u)
+// with l1 != null, the second level of the l1-ball thresholds in the same launch
 cudaError_t launch_xfield(const float *ubar, float *Fv, float *Fh, Dims dm, int grid, cudaStream_t st,
-                         int open_s, int first_order, float *Fs = nullptr);
+                         int open_s, int first_order, float *Fs = nullptr, const L1Args *l1 = nullptr);
 // SSTV's dual step: Y = clip(Y + gamma_Y D D_s ubar, -1, 1) on the cube pair
 // (Yv, Yh), and Z = Y
 cudaError_t launch_sstv_dual(const float *ubar, float *Yv, float *Yh, float *Zv, float *Zh, Dims dm, float gY,
