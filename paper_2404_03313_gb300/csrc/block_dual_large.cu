@@ -16,14 +16,17 @@
 //  2. Warm start: C0 = W G from the block's stored normalized eigen-rows W (a
 //     NaN marker in W starts cold from C0 = G).
 //  3. One-sided (Hestenes) Jacobi on the rows of C, resident in shared memory,
-//     in the round-robin ordering: each of the NPOS - 1 steps of a sweep meets
-//     NPOS / 2 disjoint row pairs, a group of 8 lanes per pair (4 where that
-//     lets one round of the warps cover a step) and 32 / group pairs per warp
-//     side by side (a dot product over the group, then the rotation of both
-//     rows, held in registers, written back in place); rows never move, only
-//     the pairing changes.  Rows are scaled by an exact
-//     power of two first; the tolerance, the numerical-zero floor and the
-//     rotation formula are those of block_dual.cu.
+//     in the round-robin ordering.  Up to 36 and from 64 rows on, two row pairs
+//     meet at a time: a group of 8 (or 16) lanes holds the four rows in registers,
+//     rotates the four pairs across the meeting and writes them back, which halves
+//     the rows moved and the barriers per sweep; in between, two rows meet, a group
+//     of 8 lanes each (4 where that lets one round of the warps cover a step).
+//     Rows never move, only the pairing changes.  Rows are scaled by an exact power
+//     of two first; the tolerance, the numerical-zero floor and the rotation formula
+//     are those of block_dual.cu, with the rotation normalized (rotation()).
+//     Measured at 100 x 100 x 198 under exact step sizes, ms per warm pass, before
+//     and now: k = 6 3.59 -> 2.45, 7 6.16 -> 4.63, 8 8.42 -> 6.10, 9 17.99 -> 17.19,
+//     10 24.75 -> 23.34 (one row pair per meeting, twice the warps per CTA).
 //  4. Converged rows are lam_x u_x^T: scaled eigen-rows into shared memory, the
 //     normalized rows into W for the next pass.
 //  5. M = I - Ut^T Ut by 4 x 4 tiles; then Y' streams through the chunk again
@@ -38,7 +41,7 @@
 // 2 x 256 x 272 floats, 557 KB per CTA; two CTAs per SM, 72 MB in all at
 // k = 13 and 165 MB at k = 16, mostly L2-resident),
 // the Gram accumulates its upper-triangle tiles over several passes of the
-// chunks (3 tiles a thread per pass) and the Jacobi uses 8-lane groups.
+// chunks (3 tiles a thread per pass) and the Jacobi uses 16-lane groups.
 // FP32 throughout (FP32 FMAs on CUDA cores).
 #include <math.h>
 #include "s3ttv_internal.cuh"
@@ -46,8 +49,7 @@
 namespace s3ttv {
 namespace {
 
-constexpr int kLW = 8;         // warps per CTA (two CTAs per SM where shared memory allows)
-constexpr int kLT = kLW * 32;  // threads per CTA
+constexpr int kLW = 8;         // warps per CTA of 65..100 and of more than 144 rows (two CTAs per SM)
 constexpr int kCW = 48;        // columns of Y' per streamed chunk
 // The Gram's 4 x 4 tiles read four chunk rows apart (4 (kCW + 4) floats, 16
 // banks mod 32) and rotate their column order within 16-column windows.
@@ -58,6 +60,17 @@ static_assert(kCW % 16 == 0 && (4 * (kCW + 4)) % 32 == 16, "chunk geometry of th
 __host__ __device__ constexpr int pair_lanes(int n, int lw) {
   return n > kMaxSmemRows ? 8
                           : (((n + 1) / 2 + lw * 8 - 1) / (lw * 8) < ((n + 1) / 2 + lw * 4 - 1) / (lw * 4) ? 4 : 8);
+}
+
+// Lanes per quad of rows in the Jacobi of step 3: 8, or 16 where the quads of a
+// step (n / 4 of them) then still fit one round of the CTA's warps, and above
+// kMaxSmemRows rows, whose four rows would not fit 8 lanes' registers.
+// Blocks of 37..63 rows keep the meetings of two rows: theirs do not divide into
+// 16-column pieces well (a stacked k = 5 sweep, 50 rows in 4 pieces, was 9% slower
+// than with 4-lane pairs).
+__host__ __device__ constexpr bool use_quads(int n) { return n <= 36 || n >= 64; }
+__host__ __device__ constexpr int quad_lanes(int n, int lw) {
+  return n > kMaxSmemRows || (n + 3) / 4 * 16 <= lw * 32 ? 16 : 8;
 }
 
 // Two FP32 values in one 64-bit register pair, and the packed FP32x2
@@ -84,6 +97,25 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
   return r;
 }
 
+// The rotation (c, s) that makes two rows of squared norms nA, nB and product d
+// orthogonal, A' = c A - s B, B' = s A + c B, and dn = t d, by which it moves the
+// squared norms apart.  tan 2 theta = 2 d / (nB - nA), |theta| <= pi / 4, from two
+// reciprocal square roots; a Newton step then brings c^2 + s^2 back to 1: they leave
+// it 1e-7 off, and a row goes through hundreds of rotations (k = 10, 200 columns: a
+// block-dual step's error 7.3e-6 without it, 3.0e-6 with it).
+__device__ __forceinline__ void rotation(float nA, float nB, float d, float &cs, float &sn, float &dn) {
+  const float x = nB - nA, y = 2.f * d;
+  const float rr = rsqrtf(fmaf(x, x, y * y));
+  const float hc = fmaf(0.5f * fabsf(x), rr, 0.5f);
+  const float rc = rsqrtf(hc);
+  cs = hc * rc;
+  sn = copysignf(0.5f, x) * y * rr * rc;
+  dn = sn * rc * d;
+  const float h = 0.5f * fmaf(-cs, cs, fmaf(-sn, sn, 1.f));
+  cs = fmaf(cs, h, cs);
+  sn = fmaf(sn, h, sn);
+}
+
 struct Layout {
   int n, npos, gs, cs;  // block rows, rows padded to even, row strides of the n x n buffers and the chunk
   int nt4;              // 4-row tiles across npos
@@ -100,10 +132,12 @@ __host__ __device__ inline Layout layout(int n, int pg) {
   L.npos = (L.n + 1) & ~1;
   L.nt4 = (L.npos + 3) / 4;
   const int w = 4 * L.nt4;  // rows and columns rounded to whole tiles
-  // a multiple of 4 (float4 rows) and 2 pg mod 32: consecutive rows start
-  // 2 pg banks apart, so the pg-lane Jacobi groups of a warp, which read
-  // neighbouring rows (2 pg floats each), fill the 32 banks without conflicts
-  L.gs = w + (2 * pg - w % 32 + 32) % 32;
+  // a multiple of 4 (float4 rows) and, for quads, 8 mod 32: the 8-lane groups of a
+  // half-warp read 64 bytes each from rows two apart, 16 banks on, and the
+  // tensor-core fragments of C0 and the apply hit distinct banks; for pairs 2 pg mod
+  // 32: consecutive rows start 2 pg banks apart, and the pg-lane groups of a warp
+  // read neighbouring rows
+  L.gs = w + ((use_quads(n) && n <= kMaxSmemRows ? 8 : 2 * pg) - w % 32 + 32) % 32;
   L.cs = kCW + 4;
   L.x1 = 0;
   L.x2 = L.x1 + (size_t)w * L.gs;
@@ -120,6 +154,8 @@ __host__ __device__ inline Layout layout(int n, int pg) {
 __device__ __forceinline__ float4 lds4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 __device__ __forceinline__ void sts4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
 __device__ __forceinline__ float c4(const float4 &v, int e) { return e == 0 ? v.x : e == 1 ? v.y : e == 2 ? v.z : v.w; }
+
+__device__ __forceinline__ void prefetch_l2(const float *p) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(p)); }
 
 // (row, column) of upper-triangle 4 x 4 tile t of an nt4 x nt4 tile grid
 __device__ __forceinline__ void upper_tile(int t, int nt4, int &ti, int &tj) {
@@ -244,21 +280,26 @@ __host__ __device__ constexpr int apply_qpu(int mt, int qt, int lw) {
   return best;
 }
 
-// warps per CTA: stacked blocks of up to 64 rows (k <= 5) and SSST's blocks
-// run four-warp CTAs, four per SM; blocks of 101..144 rows, whose two n x n
-// matrices fill one SM's shared memory, one sixteen-warp CTA per SM;
-// everything else eight-warp CTAs, two per SM
-__host__ __device__ constexpr int large_warps_for(int n_rows, bool small) {
-  return small ? 4 : (n_rows > 100 && n_rows <= kMaxSmemRows ? 16 : kLW);
+// Warps per CTA and CTAs per SM: as many warps as a Jacobi step's groups fill, and
+// as many CTAs as shared memory takes.  Up to 36 rows four-warp CTAs, eight per SM
+// (64 registers); up to 64 rows four, and up to 100 eight-warp CTAs, two per SM (128
+// registers; with 64 registers and twice the warps, 16 lanes per quad, k = 10 took
+// 29.4 ms per pass where this takes 23.6 at 100 x 100 x 198); blocks of 101..144
+// rows, whose two n x n matrices fill one SM's shared memory, one sixteen-warp CTA;
+// larger ones two eight-warp CTAs.
+__host__ __device__ constexpr int large_warps_for(int n_rows) {
+  return n_rows <= 64 ? 4 : (n_rows > 100 && n_rows <= kMaxSmemRows ? 16 : kLW);
+}
+__host__ __device__ constexpr int large_ctas(int n_rows) {
+  return n_rows <= 36 ? 8 : (n_rows <= 64 ? 4 : (n_rows > 100 && n_rows <= kMaxSmemRows ? 1 : 2));
 }
 template <int K, bool ST, int PARTS>
 __host__ __device__ constexpr int large_warps() {
-  return large_warps_for(ST ? 2 * K * K : K * K, (ST && 2 * K * K <= 64) || (PARTS == 3 && K * K <= 64));
+  return large_warps_for(ST ? 2 * K * K : K * K);
 }
 
 template <int K, bool ST, int PARTS>
-__global__ void __launch_bounds__(large_warps<K, ST, PARTS>() * 32,
-                                  large_warps<K, ST, PARTS>() == 4 ? 4 : (large_warps<K, ST, PARTS>() == 16 ? 1 : 2))
+__global__ void __launch_bounds__(large_warps<K, ST, PARTS>() * 32, large_ctas(ST ? 2 * K * K : K * K))
     block_dual_large_kernel(BlockDualArgs a) {
   chained();
   constexpr int LW = large_warps<K, ST, PARTS>(), LT = LW * 32;
@@ -270,7 +311,10 @@ __global__ void __launch_bounds__(large_warps<K, ST, PARTS>() * 32,
   constexpr int GTP = GT > 3 ? 3 : GT, NPASS = (GT + GTP - 1) / GTP;
   constexpr int SL = (NR + 31) / 32;                   // row elements a lane holds
   constexpr int PG = pair_lanes(NR, LW);               // lanes per row pair in the Jacobi
-  constexpr int PE2 = (NR + 2 * PG - 1) / (2 * PG);    // float2 pieces of a row a Jacobi lane holds
+  constexpr int PE2 = (NR + 2 * PG - 1) / (2 * PG);    // float2 pieces of a row a lane of a pair holds
+  constexpr int QL = quad_lanes(NR, LW);               // lanes per quad of rows in the Jacobi
+  constexpr int QE = (NR + 2 * QL - 1) / (2 * QL);     // float2 pieces of each row a lane of a quad holds
+  constexpr int NS = ((NR + 1) / 2 + 1) & ~1;          // row pairs, padded to an even count
   // skip Jacobi pairs whose rows are unchanged since they last met: pays from
   // about 64 rows (measured: k = 10 3% faster, SSST's 25 rows 8% slower)
   constexpr bool SKIP = NR > 64;
@@ -319,7 +363,7 @@ __global__ void __launch_bounds__(large_warps<K, ST, PARTS>() * 32,
     // chunks, measured) fetch the next chunk into registers while this one's
     // products run; larger ones would spill (two CTAs per SM) and stream as is.
     constexpr int PC = (4 * NT4 * (kCW / 4) + LT - 1) / LT;
-    constexpr bool PREF = PC <= 6 && NR < 64;
+    constexpr bool PREF = PC <= (NR <= 36 ? 3 : 6) && NR < 64;
     constexpr int PCR = PREF ? PC : 1;
     float4 ry[PCR], rf[PCR];
     if constexpr (PREF) fetch_chunk<ST, LT, PARTS, PCR>(L, Yl, a, pix, 0, ps == 0, ry, rf);
@@ -328,6 +372,8 @@ __global__ void __launch_bounds__(large_warps<K, ST, PARTS>() * 32,
         place_chunk<ST, LT, PARTS, PCR>(L, chunk, Yl, a, c0, ps == 0, ry, rf);
       } else {
         stream_chunk<ST, LT, PARTS>(L, chunk, Yl, a, pix, c0, ps == 0);
+        if (ps == 0 && c0 + kCW < W)  // the next chunk's rows on their way into L2 meanwhile
+          for (int it = tid; it < 2 * n; it += LT) prefetch_l2(Yl + (size_t)(it >> 1) * W + min(c0 + kCW + 32 * (it & 1), W - 1));
       }
       __syncthreads();
       if constexpr (PREF)
@@ -497,6 +543,11 @@ __global__ void __launch_bounds__(large_warps<K, ST, PARTS>() * 32,
     }
     __syncthreads();
 
+    // the next block's first chunk on its way into L2 while this one is solved
+    if (l + gridDim.x < Lb)
+      for (int it = tid; it < 2 * n; it += LT)
+        prefetch_l2(Yl + (size_t)gridDim.x * n * W + (size_t)(it >> 1) * W + min(32 * (it & 1), W - 1));
+
     // ---- 3. one-sided Jacobi on the rows of C ----
     if (SKIP)
       for (int r = tid; r < NP; r += LT) last[r] = -2;  // published by the barrier in norms()
@@ -538,6 +589,128 @@ __global__ void __launch_bounds__(large_warps<K, ST, PARTS>() * 32,
     for (int sw = 0; sw < a.max_sweeps; ++sw) {
       if (sw) norms();
       int rotated = 0;
+      if constexpr (use_quads(NR)) {
+      // Rows 2 s and 2 s + 1 form row pair s; the row pairs meet in round-robin
+      // order, and a group of QL lanes holds the four rows of a meeting in
+      // registers and rotates the four row pairs across it (at a sweep's first
+      // step also the two within).  Against one row pair per meeting this halves
+      // the rows loaded and stored, which bound the sweep (62k of 96k cycles per
+      // sweep and SM at n = 100 were shared-memory wavefronts), and the barriers.
+      for (int step = 0; step < NS - 1; ++step) {
+        for (int base = 0; base < NS / 2; base += LW * (32 / QL)) {
+          if (base + warp * (32 / QL) >= NS / 2) continue;  // the whole warp has no quad this round
+          const int i = base + warp * (32 / QL) + (lane / QL), gl = lane % QL;
+          const bool act = i < NS / 2;
+          // round robin: position 0 fixed, positions 1..NS-1 turn by one each step
+          const int pa = act ? i : 0, pb = NS - 1 - pa;
+          int xa = pa - 1 + step, xb = pb - 1 + step;  // both < 2 (NS - 1)
+          xa -= xa >= NS - 1 ? NS - 1 : 0;
+          xb -= xb >= NS - 1 ? NS - 1 : 0;
+          const int ra = pa == 0 ? 0 : 2 + 2 * xa, rb = 2 + 2 * xb;
+          const int row[4] = {ra, ra + 1, rb, rb + 1};
+          // a quad whose rows no rotation has touched since they last met (in the
+          // previous sweep, with the same rows, and did not rotate then) would
+          // compute the same products: it is skipped
+          bool chk = act;
+          if (SKIP && sw > 0 && act) {
+            int m = -2;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) m = row[q] < NP ? max(m, last[row[q]]) : m;
+            chk = m >= sw - 1;
+          }
+          if (!__any_sync(kFull, chk)) continue;  // warp-uniform
+          // lane gl holds the float2 pieces at columns 2 gl + 2 QL e; columns
+          // n..GS-1 of every row are zero, so a piece starting below n is whole
+          f32x2 v[4][QE];
+          float nr[4];
+          bool dirty[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const bool in = chk && row[q] < NP;  // (rows of the padding pair are zero)
+            const float *R = X2 + (size_t)row[q] * GS;
+            nr[q] = in ? nrm[row[q]] : 0.f;
+            dirty[q] = false;
+#pragma unroll
+            for (int e = 0; e < QE; ++e) {
+              const int c = 2 * gl + 2 * QL * e;
+              v[q][e] = in && c < n ? *reinterpret_cast<const f32x2 *>(R + c) : 0ull;
+            }
+          }
+          // Rotate rows (p0, q0) and (p1, q1), two disjoint pairs, where they need
+          // it.  The lower half of the group reduces the first pair's product and
+          // works out its rotation, the upper half the second's, in one
+          // instruction stream; then they trade.
+          auto rotate2 = [&](auto P0, auto Q0, auto P1, auto Q1) {
+            constexpr int p0 = decltype(P0)::value, q0 = decltype(Q0)::value;
+            constexpr int p1 = decltype(P1)::value, q1 = decltype(Q1)::value;
+            f32x2 da = 0ull, db = 0ull;
+#pragma unroll
+            for (int e = 0; e < QE; ++e) {
+              da = fma2(v[p0][e], v[q0][e], da);
+              db = fma2(v[p1][e], v[q1][e], db);
+            }
+            const float2 fa = up2(da), fb = up2(db);
+            const float s0 = fa.x + fa.y, s1 = fb.x + fb.y;
+            const bool hi = gl >= QL / 2;
+            float d = (hi ? s1 : s0) + __shfl_xor_sync(kFull, hi ? s0 : s1, QL / 2);
+#pragma unroll
+            for (int o = QL / 4; o > 0; o >>= 1) d += __shfl_xor_sync(kFull, d, o);
+            const float nA = hi ? nr[p1] : nr[p0], nB = hi ? nr[q1] : nr[q0];
+            const bool need = fminf(nA, nB) > floor2 && d * d > pol2 * nA * nB;
+            if (!__any_sync(kFull, need)) return;
+            float cs = 1.f, sn = 0.f, dn = 0.f;
+            if (need) {
+              rotation(nA, nB, d, cs, sn, dn);
+              if (d * d > tol2 * nA * nB) rotated = 1;
+            }
+            const float cso = __shfl_xor_sync(kFull, cs, QL / 2), sno = __shfl_xor_sync(kFull, sn, QL / 2);
+            const float dno = __shfl_xor_sync(kFull, dn, QL / 2);
+            auto apply = [&](f32x2(&A)[QE], f32x2(&B)[QE], float c, float sv) {
+              const f32x2 cs2 = pk2(c, c), sn2 = pk2(sv, sv), ns2 = pk2(-sv, -sv);
+#pragma unroll
+              for (int e = 0; e < QE; ++e) {
+                const f32x2 va = A[e], vb = B[e];
+                A[e] = fma2(cs2, va, mul2(ns2, vb));
+                B[e] = fma2(sn2, va, mul2(cs2, vb));
+              }
+            };
+            const float sa = hi ? sno : sn, sb = hi ? sn : sno;
+            apply(v[p0], v[q0], hi ? cso : cs, sa);
+            apply(v[p1], v[q1], hi ? cs : cso, sb);
+            const float na = hi ? dno : dn, nb2 = hi ? dn : dno;
+            nr[p0] -= na;
+            nr[q0] += na;
+            nr[p1] -= nb2;
+            nr[q1] += nb2;
+            if (sa != 0.f) dirty[p0] = dirty[q0] = true;
+            if (sb != 0.f) dirty[p1] = dirty[q1] = true;
+          };
+          using I0 = std::integral_constant<int, 0>;
+          using I1 = std::integral_constant<int, 1>;
+          using I2 = std::integral_constant<int, 2>;
+          using I3 = std::integral_constant<int, 3>;
+          if (step == 0) rotate2(I0{}, I1{}, I2{}, I3{});
+          rotate2(I0{}, I2{}, I1{}, I3{});
+          rotate2(I0{}, I3{}, I1{}, I2{});
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if (!dirty[q]) continue;
+            float *R = X2 + (size_t)row[q] * GS;
+#pragma unroll
+            for (int e = 0; e < QE; ++e) {
+              const int c = 2 * gl + 2 * QL * e;
+              if (c < n) *reinterpret_cast<f32x2 *>(R + c) = v[q][e];
+            }
+            if (gl == 0) {
+              nrm[row[q]] = nr[q];
+              if (SKIP) last[row[q]] = sw;
+            }
+          }
+        }
+        __syncthreads();
+      }
+      } else {
+      // one meeting of two rows per group of PG lanes
       for (int step = 0; step < NP - 1; ++step) {
         // PG lanes per pair, 32 / PG pairs per warp side by side
         for (int base = 0; base < NP / 2; base += LW * (32 / PG)) {
@@ -574,12 +747,8 @@ __global__ void __launch_bounds__(large_warps<K, ST, PARTS>() * 32,
           for (int o = PG / 2; o > 0; o >>= 1) d += __shfl_xor_sync(kFull, d, o);
           const float nA = chk ? nrm[ra] : 0.f, nB = chk ? nrm[rb] : 0.f;
           if (chk && fminf(nA, nB) > floor2 && d * d > pol2 * nA * nB) {
-            const float x = nB - nA, y = 2.f * d;
-            const float rr = rsqrtf(fmaf(x, x, y * y));
-            const float hc = fmaf(0.5f * fabsf(x), rr, 0.5f);
-            const float rc = rsqrtf(hc);
-            const float cs = hc * rc, sn = copysignf(0.5f, x) * y * rr * rc;
-            const float dn = sn * rc * d;  // t apq
+            float cs, sn, dn;
+            rotation(nA, nB, d, cs, sn, dn);
             const f32x2 cs2 = pk2(cs, cs), sn2 = pk2(sn, sn), ns2 = pk2(-sn, -sn);
 #pragma unroll
             for (int e = 0; e < PE2; ++e) {
@@ -601,6 +770,7 @@ __global__ void __launch_bounds__(large_warps<K, ST, PARTS>() * 32,
           }
         }
         __syncthreads();
+      }
       }
       ++sweeps;
       if (!__syncthreads_or(rotated)) {
@@ -917,8 +1087,16 @@ __global__ void __launch_bounds__(large_warps<K, ST, PARTS>() * 32,
       constexpr int QPU = apply_qpu(MT, QT, LW), UPR = QT / QPU, UNITS = MT * UPR;
       constexpr int ROUNDS = (UNITS + LW - 1) / LW;
       const int g = lane >> 2, t = lane & 3;
+      // the next chunk of Y' is fetched into registers (free by then) while this
+      // one's results are stored and added into Z
+      constexpr int PCA = (4 * NT4 * (kCW / 4) + LT - 1) / LT;
+      constexpr bool PREFA = PCA <= 6;
+      constexpr int PCAR = PREFA ? PCA : 1;
+      float4 ry[PCAR], rf[PCAR];
+      if constexpr (PREFA) fetch_chunk<ST, LT, PARTS, PCAR>(L, Yl, a, pix, 0, false, ry, rf);
       for (int c0 = 0; c0 < W; c0 += kCW) {
-        stream_chunk<ST, LT, PARTS>(L, chunk, Yl, a, pix, c0, false);
+        if constexpr (PREFA) place_chunk<ST, LT, PARTS, PCAR>(L, chunk, Yl, a, c0, false, ry, rf);
+        else stream_chunk<ST, LT, PARTS>(L, chunk, Yl, a, pix, c0, false);
         __syncthreads();
         // unit u: rows 16 m .. 16 m + 15 of the chunk's result, QPU column tiles of 8
         float d[ROUNDS][QPU][4];
@@ -971,6 +1149,8 @@ __global__ void __launch_bounds__(large_warps<K, ST, PARTS>() * 32,
             }
         }
         __syncthreads();
+        if constexpr (PREFA)
+          if (c0 + kCW < W) fetch_chunk<ST, LT, PARTS, PCAR>(L, Yl, a, pix, c0 + kCW, false, ry, rf);
         constexpr int Q = kCW / 4;
         for (int it = tid; it < n * Q; it += LT) {
           const int r = it / Q, j = it - r * Q, c = c0 + 4 * j;
@@ -1009,9 +1189,9 @@ long long block_dual_large_w_stride(int k, bool stacked) {
 
 long long block_dual_large_w_stride(int k) { return block_dual_large_w_stride(k, false); }
 
-int block_dual_large_threads(int k, bool stacked, int parts) {
+int block_dual_large_threads(int k, bool stacked, int) {
   const int n = stacked ? 2 * k * k : k * k;
-  return 32 * large_warps_for(n, (stacked && n <= 64) || (parts == 3 && k * k <= 64));
+  return 32 * large_warps_for(n);
 }
 
 namespace {
