@@ -28,13 +28,11 @@
 //    concatenation of a half-size tensor read through nearest upsampling and a
 //    same-size one.  The input gradient is the same kernel with the output
 //    gradient as input and the weights transposed and mirrored.
-//  * conv_wgrad_kernel: dW[o, tap, c] = sum_p G[p, o] X[p + delta_tap, c]:
-//    M = output channels, N = 32 input channels of one tap, K = voxels of one
-//    chunk; fragments come from the voxel-major tiles through ldmatrix.trans;
-//    partial sums are added into FP32 dW with atomics.
+//    So are the weight gradients, with the voxels as the K dimension and partial
+//    sums added into FP32 dW with atomics (unet_conv.cu).
 //  * the first layer (one input channel) and the head run on CUDA cores; the
-//    first layer's weight gradient goes through an im2col of its 27 taps and
-//    the tensor-core weight-gradient kernel.
+//    first layer's weight gradient goes through an im2col of its 27 taps and a
+//    small mma.sync kernel.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -152,106 +150,42 @@ __device__ __forceinline__ void store8(bf16 *p, const float f[8]) {
   *reinterpret_cast<uint4 *>(p) = u;
 }
 
-// ---------------------------------------------------------------- weight gradient
-constexpr int kBK = 32;     // input channels per CTA
+// ---------------------------------------------------------------- first layer's weight gradient
+// dW[o][j] = sum_p G[p, o] N[p, j] with N the 27 neighbour values of every voxel and a
+// one (im2col_first_kernel): 32 x 32 outputs over one chunk of voxels per CTA in
+// stages of kWS, four warps of 16 x 16 (mma.sync; the other layers' weight gradients
+// run in unet_conv.cu).
 constexpr int kAS = 40;     // shared row stride in bf16 (80 B: ldmatrix rows hit distinct banks)
 constexpr int kStages = 3;  // cp.async pipeline depth
+constexpr int kWS = 64;     // voxels per stage
+constexpr int kFirstSmem = kStages * kWS * 2 * kAS * (int)sizeof(bf16);
 
-struct WgradArgs {
-  const bf16 *g;    // [V][cout] output gradient (ReLU mask applied)
-  const bf16 *x0;
-  const bf16 *x1;
-  float *dw;        // [cout][27][c1 + c0], accumulated
-  int c0, c1, cout, chunk;
-  int first;        // 1: x0 holds the first layer's 27 neighbour values per voxel (+5 zeros); one
-                    // unshifted "tap", output dw[o][j] for j < 27
-  Vol vol;
-};
-
-constexpr int kWS = 64;  // voxels per weight-gradient stage
-
-template <int MT>
-constexpr int wgrad_smem_bytes() {
-  return kStages * kWS * ((MT + 8) + kAS) * (int)sizeof(bf16);
-}
-
-// CTA: MT output channels x 32 input channels of one tap, over one chunk of
-// voxels in stages of kWS; four warps, each (MT / 2) x 16.
-template <int MT>
-__global__ void __launch_bounds__(128) conv_wgrad_kernel(WgradArgs a) {
-  constexpr int GS = MT + 8;  // shared row stride of the gradient tile (bf16)
-  constexpr int GE = kWS * GS, XE = kWS * kAS;
+__global__ void __launch_bounds__(128) wgrad_first_kernel(const bf16 *G, const bf16 *N, float *dw, float *db, int V,
+                                                          int chunk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   bf16 *Gs = reinterpret_cast<bf16 *>(smem_raw);
-  bf16 *Xs = Gs + kStages * GE;
+  bf16 *Xs = Gs + kStages * kWS * kAS;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int wm = warp & 1, wn = warp >> 1;
-  const int cin = a.c0 + a.c1, nch = cin / kBK;
-  const int tap = a.first ? 13 : blockIdx.x / nch, cb = (blockIdx.x - (a.first ? 0 : tap) * nch) * kBK;
-  const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-  const int co0 = blockIdx.y * MT;
-  const Vol &g = a.vol;
-  const int V = nvox(g);
-  const int pbeg = blockIdx.z * a.chunk, pend = min(V, pbeg + a.chunk);
+  const int pbeg = blockIdx.x * chunk, pend = min(V, pbeg + chunk);
   if (pbeg >= pend) return;
   const int nst = (pend - pbeg + kWS - 1) / kWS;
-  const int off0 = (dz * g.H + dy) * g.W + dx;
-  const int D2 = g.D >> 1, H2 = g.H >> 1, W2 = g.W >> 1;
-
-  // the two X rows this thread gathers (r0, r0 + 32), advanced by kWS per stage
-  const int r0 = tid >> 2, xq = tid & 3;
-  int vb[2], vz[2], vy[2], vx[2];
-#pragma unroll
-  for (int i = 0; i < 2; ++i) decode(min(pbeg + r0 + 32 * i, V - 1), g, vb[i], vz[i], vy[i], vx[i]);
+  const int r0 = tid >> 2, q = tid & 3;
   auto load = [&](int st, int buf) {
-    const int pb = pbeg + st * kWS;
-    bf16 *gs = Gs + buf * GE;
-#pragma unroll
-    for (int i = 0; i < MT / 16; ++i) {
-      const int e = tid + 128 * i;
-      const int r = e / (MT / 8), qq = e % (MT / 8);
-      const int p = pb + r;
-      const bool ok = p < pend;
-      cp_async16(gs + r * GS + qq * 8, ok ? a.g + (size_t)p * a.cout + co0 + qq * 8 : a.g, ok ? 16 : 0);
-    }
-    bf16 *xs = Xs + buf * XE;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      const int r = r0 + 32 * i, p = pb + r;
-      const int z = vz[i] + dz, y = vy[i] + dy, x = vx[i] + dx;
-      const bool ok = p < pend && z >= 0 && z < g.D && y >= 0 && y < g.H && x >= 0 && x < g.W;
-      const bf16 *src = a.g;
-      if (ok) {
-        if (cb < a.c1)
-          src = a.x1 + (size_t)(unsigned)(((vb[i] * D2 + (z >> 1)) * H2 + (y >> 1)) * W2 + (x >> 1)) * a.c1 + cb +
-                xq * 8;
-        else
-          src = a.x0 + (size_t)(unsigned)(p + off0) * a.c0 + (cb - a.c1) + xq * 8;
-      }
-      cp_async16(xs + r * kAS + xq * 8, src, ok ? 16 : 0);
-      vx[i] += kWS;
-      while (vx[i] >= g.W) {
-        vx[i] -= g.W;
-        if (++vy[i] == g.H) {
-          vy[i] = 0;
-          if (++vz[i] == g.D) {
-            vz[i] = 0;
-            ++vb[i];
-          }
-        }
-      }
+      const int r = r0 + 32 * i, p = pbeg + st * kWS + r;
+      const bool ok = p < pend;
+      const size_t o = (size_t)(ok ? p : pbeg) * 32 + q * 8;
+      cp_async16(Gs + (buf * kWS + r) * kAS + q * 8, G + o, ok ? 16 : 0);
+      cp_async16(Xs + (buf * kWS + r) * kAS + q * 8, N + o, ok ? 16 : 0);
     }
   };
-
-  constexpr int MI = MT / 32;  // m16 tiles per warp (the warp owns MT / 2 rows)
-  float acc[MI][2][4];
+  float acc[2][4];
 #pragma unroll
-  for (int i = 0; i < MI; ++i)
+  for (int j = 0; j < 2; ++j)
 #pragma unroll
-    for (int j = 0; j < 2; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
-
+    for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
 #pragma unroll
   for (int st = 0; st < kStages - 1; ++st) {
     if (st < nst) load(st, st);
@@ -263,176 +197,24 @@ __global__ void __launch_bounds__(128) conv_wgrad_kernel(WgradArgs a) {
     __syncthreads();
     if (st + kStages - 1 < nst) load(st + kStages - 1, (st + kStages - 1) % kStages);
     cp_async_commit();
-    const bf16 *gs = Gs + (st % kStages) * GE, *xs = Xs + (st % kStages) * XE;
+    const bf16 *gs = Gs + (st % kStages) * kWS * kAS, *xs = Xs + (st % kStages) * kWS * kAS;
 #pragma unroll
     for (int kk = 0; kk < kWS; kk += 16) {
-      uint32_t bfr[4];  // B[k = voxel][n = channel] from Xs[k][n], transposed on load
+      uint32_t af[4], bfr[4];  // A[m = out channel][k = voxel], B[k][n = neighbour], transposed on load
       ldsm_x4_t(bfr, xs + (kk + (mat & 1) * 8 + r8) * kAS + wn * 16 + (mat >> 1) * 8);
-#pragma unroll
-      for (int mi = 0; mi < MI; ++mi) {
-        uint32_t af[4];  // A[m = out channel][k = voxel] from Gs[k][m], transposed on load
-        ldsm_x4_t(af, gs + (kk + (mat >> 1) * 8 + r8) * GS + wm * (MT / 2) + mi * 16 + (mat & 1) * 8);
-        mma_bf16(acc[mi][0], af, bfr[0], bfr[1]);
-        mma_bf16(acc[mi][1], af, bfr[2], bfr[3]);
-      }
+      ldsm_x4_t(af, gs + (kk + (mat >> 1) * 8 + r8) * kAS + wm * 16 + (mat & 1) * 8);
+      mma_bf16(acc[0], af, bfr[0], bfr[1]);
+      mma_bf16(acc[1], af, bfr[2], bfr[3]);
     }
   }
-
   const int gq = lane >> 2, t4 = lane & 3;
 #pragma unroll
-  for (int mi = 0; mi < MI; ++mi)
+  for (int nj = 0; nj < 2; ++nj)
 #pragma unroll
-    for (int nj = 0; nj < 2; ++nj)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int o = co0 + wm * (MT / 2) + mi * 16 + gq + 8 * (e >> 1);
-        const int c = cb + wn * 16 + nj * 8 + 2 * t4 + (e & 1);
-        if (a.first) {
-          if (c < 27) atomicAdd(a.dw + o * 27 + c, acc[mi][nj][e]);
-        } else {
-          atomicAdd(a.dw + ((size_t)o * 27 + tap) * cin + c, acc[mi][nj][e]);
-        }
-      }
-}
-
-template <int MT>
-constexpr int wgrad4_smem_bytes() {
-  return kStages * kWS * ((MT + 8) + 4 * kAS) * (int)sizeof(bf16);
-}
-
-// Four taps per CTA: warp w owns tap 4 t + w (t = blockIdx.x / nch) for all MT
-// output channels x 32 input channels, so the gradient tile of a stage is
-// shared by four warps and each warp runs (MT / 16) x 4 fragments per 16 voxels.
-template <int MT>
-__global__ void __launch_bounds__(128) conv_wgrad4_kernel(WgradArgs a) {
-  constexpr int GS = MT + 8;
-  constexpr int GE = kWS * GS, XE = kWS * kAS;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  bf16 *Gs = reinterpret_cast<bf16 *>(smem_raw);
-  bf16 *Xs = Gs + kStages * GE;  // [stage][tap][voxel][channel]
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int cin = a.c0 + a.c1, nch = cin / kBK;
-  const int tg = blockIdx.x / nch, cb = (blockIdx.x - tg * nch) * kBK;
-  const int co0 = blockIdx.y * MT;
-  const Vol &g = a.vol;
-  const int V = nvox(g);
-  const int pbeg = blockIdx.z * a.chunk, pend = min(V, pbeg + a.chunk);
-  if (pbeg >= pend) return;
-  const int nst = (pend - pbeg + kWS - 1) / kWS;
-  const int D2 = g.D >> 1, H2 = g.H >> 1, W2 = g.W >> 1;
-  int tdz[4], tdy[4], tdx[4], toff[4];
-  bool tv[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int t = 4 * tg + j;
-    tv[j] = t < 27;
-    tdz[j] = t / 9 - 1;
-    tdy[j] = (t / 3) % 3 - 1;
-    tdx[j] = t % 3 - 1;
-    toff[j] = (tdz[j] * g.H + tdy[j]) * g.W + tdx[j];
-  }
-
-  const int r0 = tid >> 2, xq = tid & 3;
-  int vb[2], vz[2], vy[2], vx[2];
-#pragma unroll
-  for (int i = 0; i < 2; ++i) decode(min(pbeg + r0 + 32 * i, V - 1), g, vb[i], vz[i], vy[i], vx[i]);
-  auto load = [&](int st, int buf) {
-    const int pb = pbeg + st * kWS;
-    bf16 *gs = Gs + buf * GE;
-#pragma unroll
-    for (int i = 0; i < MT / 16; ++i) {
-      const int e = tid + 128 * i;
-      const int r = e / (MT / 8), qq = e % (MT / 8);
-      const int p = pb + r;
-      const bool ok = p < pend;
-      cp_async16(gs + r * GS + qq * 8, ok ? a.g + (size_t)p * a.cout + co0 + qq * 8 : a.g, ok ? 16 : 0);
+    for (int e = 0; e < 4; ++e) {
+      const int o = wm * 16 + gq + 8 * (e >> 1), c = wn * 16 + nj * 8 + 2 * t4 + (e & 1);
+      if (c <= 27) atomicAdd(c < 27 ? dw + o * 27 + c : db + o, acc[nj][e]);
     }
-    bf16 *xs = Xs + buf * 4 * XE;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int r = r0 + 32 * i, p = pb + r;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int z = vz[i] + tdz[j], y = vy[i] + tdy[j], x = vx[i] + tdx[j];
-        const bool ok = tv[j] && p < pend && z >= 0 && z < g.D && y >= 0 && y < g.H && x >= 0 && x < g.W;
-        const bf16 *src = a.g;
-        if (ok) {
-          if (cb < a.c1)
-            src = a.x1 + (size_t)(unsigned)(((vb[i] * D2 + (z >> 1)) * H2 + (y >> 1)) * W2 + (x >> 1)) * a.c1 + cb +
-                  xq * 8;
-          else
-            src = a.x0 + (size_t)(unsigned)(p + toff[j]) * a.c0 + (cb - a.c1) + xq * 8;
-        }
-        cp_async16(xs + j * XE + r * kAS + xq * 8, src, ok ? 16 : 0);
-      }
-      vx[i] += kWS;
-      while (vx[i] >= g.W) {
-        vx[i] -= g.W;
-        if (++vy[i] == g.H) {
-          vy[i] = 0;
-          if (++vz[i] == g.D) {
-            vz[i] = 0;
-            ++vb[i];
-          }
-        }
-      }
-    }
-  };
-
-  constexpr int MI = MT / 16;
-  float acc[MI][4][4];
-#pragma unroll
-  for (int i = 0; i < MI; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
-
-#pragma unroll
-  for (int st = 0; st < kStages - 1; ++st) {
-    if (st < nst) load(st, st);
-    cp_async_commit();
-  }
-  const int mat = lane >> 3, r8 = lane & 7;
-  const bool active = 4 * tg + warp < 27;
-  for (int st = 0; st < nst; ++st) {
-    cp_async_wait1();
-    __syncthreads();
-    if (st + kStages - 1 < nst) load(st + kStages - 1, (st + kStages - 1) % kStages);
-    cp_async_commit();
-    if (!active) continue;
-    const bf16 *gs = Gs + (st % kStages) * GE, *xs = Xs + ((st % kStages) * 4 + warp) * XE;
-#pragma unroll
-    for (int kk = 0; kk < kWS; kk += 16) {
-      uint32_t bfr[2][4];
-#pragma unroll
-      for (int nj2 = 0; nj2 < 2; ++nj2)
-        ldsm_x4_t(bfr[nj2], xs + (kk + (mat & 1) * 8 + r8) * kAS + nj2 * 16 + (mat >> 1) * 8);
-#pragma unroll
-      for (int mi = 0; mi < MI; ++mi) {
-        uint32_t af[4];
-        ldsm_x4_t(af, gs + (kk + (mat >> 1) * 8 + r8) * GS + mi * 16 + (mat & 1) * 8);
-#pragma unroll
-        for (int nj2 = 0; nj2 < 2; ++nj2) {
-          mma_bf16(acc[mi][2 * nj2], af, bfr[nj2][0], bfr[nj2][1]);
-          mma_bf16(acc[mi][2 * nj2 + 1], af, bfr[nj2][2], bfr[nj2][3]);
-        }
-      }
-    }
-  }
-  if (!active) return;
-  const int tap = 4 * tg + warp;
-  const int gq = lane >> 2, t4 = lane & 3;
-#pragma unroll
-  for (int mi = 0; mi < MI; ++mi)
-#pragma unroll
-    for (int nj = 0; nj < 4; ++nj)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int o = co0 + mi * 16 + gq + 8 * (e >> 1);
-        const int c = cb + nj * 8 + 2 * t4 + (e & 1);
-        atomicAdd(a.dw + ((size_t)o * 27 + tap) * cin + c, acc[mi][nj][e]);
-      }
 }
 
 // ---------------------------------------------------------------- first layer (one input channel)
@@ -497,8 +279,8 @@ __global__ void __launch_bounds__(256, 2) conv_first_kernel(const float *v, cons
   }
 }
 
-// col[p][j] = v[p + delta_j] for the 27 taps j (zero outside the volume), then
-// five zeros: the first layer's input as 32 BF16 channels, so its weight
+// col[p][j] = v[p + delta_j] for the 27 taps j (zero outside the volume), a one (so
+// that column 27 of the weight gradient is the bias gradient) and four zeros: the first layer's input as 32 BF16 channels, so its weight
 // gradient runs on the tensor-core weight-gradient kernel.
 __global__ void __launch_bounds__(256) im2col_first_kernel(const float *v, bf16 *col, Vol g) {
   const int V = nvox(g);
@@ -508,7 +290,7 @@ __global__ void __launch_bounds__(256) im2col_first_kernel(const float *v, bf16 
     float nb[32];
 #pragma unroll
     for (int t = 0; t < 32; ++t) {
-      nb[t] = 0.f;
+      nb[t] = t == 27 ? 1.f : 0.f;
       if (t < 27) {
         const int zz = z + t / 9 - 1, y2 = y + (t / 3) % 3 - 1, x2 = x + t % 3 - 1;
         if (zz >= 0 && zz < g.D && y2 >= 0 && y2 < g.H && x2 >= 0 && x2 < g.W)
@@ -517,22 +299,6 @@ __global__ void __launch_bounds__(256) im2col_first_kernel(const float *v, bf16 
     }
 #pragma unroll
     for (int c8 = 0; c8 < 4; ++c8) store8(col + (size_t)p * 32 + c8 * 8, nb + 8 * c8);
-  }
-}
-
-// ---------------------------------------------------------------- bias gradient
-// out[c] += sum_p G[p][c] over one chunk of voxels (C divides 256).
-__global__ void __launch_bounds__(256) colsum_kernel(const bf16 *G, int V, int C, int chunk, float *out) {
-  __shared__ float red[256];
-  const int c = threadIdx.x % C, r0 = threadIdx.x / C, R = 256 / C;
-  const int pbeg = blockIdx.x * chunk, pend = min(V, pbeg + chunk);
-  float s = 0.f;
-  for (int p = pbeg + r0; p < pend; p += R) s += __bfloat162float(G[(size_t)p * C + c]);
-  red[threadIdx.x] = s;
-  __syncthreads();
-  if (r0 == 0) {
-    for (int r = 1; r < R; ++r) s += red[r * C + c];
-    atomicAdd(out + c, s);
   }
 }
 
@@ -799,35 +565,9 @@ cudaError_t launch_conv(const s3ttv_net *net, const bf16 *x0, int c0, const bf16
 }
 
 cudaError_t launch_wgrad(const s3ttv_net *net, const bf16 *G, int cout, const bf16 *x0, int c0, const bf16 *x1,
-                         int c1, float *dw, Vol g) {
-  const int V = nvox(g);
-  // up to 64 output channels: four taps per CTA; 128: one tap per CTA
-  const bool four = cout <= 64;
-  const int MT = four ? cout : 128;
-  const int gx = (four ? 7 : 27) * ((c0 + c1) / kBK), gy = cout / MT;
-  const long long target = (long long)net->num_sms * 8;
-  long long z = (target + (long long)gx * gy - 1) / ((long long)gx * gy);
-  const long long zmax = (V + 511) / 512;
-  if (z > zmax) z = zmax;
-  if (z < 1) z = 1;
-  int chunk = (int)(((V + z - 1) / z + kWS - 1) / kWS * kWS);
-  z = (V + chunk - 1) / chunk;
-  WgradArgs a{G, x0, x1, dw, c0, c1, cout, chunk, 0, g};
-  dim3 grid(gx, gy, (unsigned)z);
-  if (MT == 128)
-    conv_wgrad_kernel<128><<<grid, 128, wgrad_smem_bytes<128>(), net->stream>>>(a);
-  else if (MT == 64)
-    conv_wgrad4_kernel<64><<<grid, 128, wgrad4_smem_bytes<64>(), net->stream>>>(a);
-  else
-    conv_wgrad4_kernel<32><<<grid, 128, wgrad4_smem_bytes<32>(), net->stream>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_colsum(const s3ttv_net *net, const bf16 *G, int V, int C, float *out) {
-  const int blocks = grid_for(net, V, 256);
-  const int chunk = (V + blocks - 1) / blocks;
-  colsum_kernel<<<(V + chunk - 1) / chunk, 256, 0, net->stream>>>(G, V, C, chunk, out);
-  return cudaGetLastError();
+                         int c1, float *dw, float *db, Vol g) {
+  WgradTcArgs a{G, x0, x1, dw, db, c0, c1, cout, g, net->err_flag};
+  return wgrad_launch(a, net->num_sms, net->stream);
 }
 
 Vol half(const Vol &g) { return Vol{g.B, g.D / 2, g.H / 2, g.W / 2}; }
@@ -958,9 +698,7 @@ int run_backward(s3ttv_net *net, const float *v, const float *tu, const float *t
                                                                    net->gB0, G + T.hw_off, net->loss);
   NCU(cudaGetLastError());
   auto wgrad = [&](int l, const bf16 *gout, const bf16 *x0, int c0, const bf16 *x1, int c1, const Vol &g) {
-    cudaError_t e = launch_wgrad(net, gout, T.cout[l], x0, c0, x1, c1, G + T.woff[l], g);
-    if (e == cudaSuccess) e = launch_colsum(net, gout, nvox(g), T.cout[l], G + T.boff[l]);
-    return e;
+    return launch_wgrad(net, gout, T.cout[l], x0, c0, x1, c1, G + T.woff[l], G + T.boff[l], g);
   };
   // d1b: gB0 -> gC0 (masked by d1a)
   NCU(wgrad(9, net->gB0, net->d1a, 32, nullptr, 0, g0));
@@ -1006,16 +744,11 @@ int run_backward(s3ttv_net *net, const float *v, const float *tu, const float *t
   im2col_first_kernel<<<grid_for(net, V0, 256), 256, 0, net->stream>>>(v, net->gA0, g0);
   NCU(cudaGetLastError());
   {
-    const long long target = (long long)net->num_sms * 8;
-    long long z = target;
-    const long long zmax = (V0 + 511) / 512;
-    if (z > zmax) z = zmax;
-    int chunk = (int)(((V0 + z - 1) / z + kWS - 1) / kWS * kWS);
-    z = (V0 + chunk - 1) / chunk;
-    WgradArgs wa{net->gC0, net->gA0, nullptr, G + T.woff[0], 32, 0, 32, chunk, 1, g0};
-    conv_wgrad_kernel<32><<<dim3(1, 1, (unsigned)z), 128, wgrad_smem_bytes<32>(), net->stream>>>(wa);
+    const int ctas = net->num_sms * 2;
+    const int chunk = ((V0 + ctas - 1) / ctas + kWS - 1) / kWS * kWS;
+    wgrad_first_kernel<<<(V0 + chunk - 1) / chunk, 128, kFirstSmem, net->stream>>>(net->gC0, net->gA0, G + T.woff[0],
+                                                                                   G + T.boff[0], V0, chunk);
     NCU(cudaGetLastError());
-    NCU(launch_colsum(net, net->gC0, V0, 32, G + T.boff[0]));
   }
   return S3TTV_OK;
 }
@@ -1097,17 +830,7 @@ int s3ttv_net_create(s3ttv_net **out, int device, void *stream) {
     return S3TTV_ENOMEM;
   }
   *net->err_flag = 0;
-  if (conv_prepare() != cudaSuccess ||
-      cudaFuncSetAttribute(conv_wgrad_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           wgrad_smem_bytes<128>()) != cudaSuccess ||
-      cudaFuncSetAttribute(conv_wgrad_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           wgrad_smem_bytes<64>()) != cudaSuccess ||
-      cudaFuncSetAttribute(conv_wgrad_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           wgrad_smem_bytes<32>()) != cudaSuccess ||
-      cudaFuncSetAttribute(conv_wgrad4_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           wgrad4_smem_bytes<64>()) != cudaSuccess ||
-      cudaFuncSetAttribute(conv_wgrad4_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           wgrad4_smem_bytes<32>()) != cudaSuccess) {
+  if (conv_prepare() != cudaSuccess || wgrad_prepare() != cudaSuccess) {
     cudaGetLastError();
     s3ttv_net_destroy(net);
     return S3TTV_ECUDA;

@@ -547,6 +547,225 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
   if (tid == 0 && *stop) *reinterpret_cast<volatile int *>(a.err) = 1;
 }
 
+// ---------------------------------------------------------------- weight gradient
+// dW[o, tap, c] = sum_p G[p, o] X[p + delta_tap, c] for 32 input channels (a slice)
+// and 32 output channels per CTA: the voxels are the K dimension, so both operands
+// are read voxel-major (MN-major descriptors: a core matrix is 8 voxels of x by 8
+// channels, the layout of the forward kernel's planes).  M = 128 rows are the slice's
+// channels of the planes z - 1, z and z + 1 of X and a fourth plane whose first channel
+// is one everywhere; N = 32 are the output channels of plane z of G.  One tcgen05.mma
+// per 16 voxels thus covers the taps dz = -1, 0, +1 of one (dy, dx), and its row 96 sums
+// G: the bias gradient comes along.  The 27 x 32 x 32 gradients stay in TMEM, nine
+// accumulators of 32 columns, over all of a CTA's bricks (8 x 16 voxels of one plane),
+// and are then added into dW, 32 consecutive channels per instruction.
+// Bound by the 40 cycles that M = 128, N = 32, K = 16 takes (its operand reads).  Against
+// the mma.sync kernels and column sums that it replaces (a tap per warp, every tap
+// gathering X again), four 32^3 crops, a layer with its bias gradient: 32 -> 32 at 32^3
+// 71 us before, 24 now; 96 -> 32 185 and 47; 192 -> 64 at 16^3 86 and 29; 64 -> 64 46 and 16
+// (the training gradient 1080 -> 690 us).
+constexpr int kWX = (kPX * (kTY + 2) + 6) * 16;         // bytes of a plane's 8-channel piece of X (padded: 2 mod 8 pieces)
+constexpr int kWG = (kTX * kTY + 2) * 16;               // and of G
+constexpr int kWStage = 4 * 4 * kWX + 4 * kWG;
+constexpr int kWStages = 4;
+constexpr int kWThreads = (kLoadWarps + 1) * 32;        // 8 loading warps (the first four also write the result), 1 for the MMAs
+
+struct WPlan {
+  int nsl, nt;         // slices of input channels, tiles of output channels
+  int per;             // CTAs per (slice, tile)
+  int tx, ty;          // bricks along x, y
+  int bricks;
+};
+
+__global__ void __launch_bounds__(kWThreads, 1) wgrad_tc_kernel(WgradTcArgs a, WPlan pl) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ __align__(8) uint64_t bars[2 * kWStages + 1];
+  __shared__ uint32_t s_tmem;
+  __shared__ int s_stop;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const Vol g = a.vol;
+  const int combo = blockIdx.x % (pl.nsl * pl.nt), first = blockIdx.x / (pl.nsl * pl.nt);
+  const int sl = combo % pl.nsl, nt = combo / pl.nsl;
+  const uint32_t base = smem_u32(smem), bar0 = smem_u32(bars);
+  auto full = [&](int s) { return bar0 + 8u * s; };
+  auto empty = [&](int s) { return bar0 + 8u * (kWStages + s); };
+  const uint32_t done = bar0 + 8u * (2 * kWStages);
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&s_tmem)),
+                 "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+  }
+  if (tid == kLoadWarps * 32) {
+    for (int s = 0; s < kWStages; ++s) {
+      mbar_init(full(s), kLoadWarps);
+      mbar_init(empty(s), 1);
+    }
+    mbar_init(done, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    s_stop = 0;
+  }
+  // the fourth plane of every stage: channel 0 one, the others zero
+  for (int i = tid; i < kWStages * 4 * (kWX / 16); i += kWThreads) {
+    const int st = i / (4 * (kWX / 16)), e = i - st * 4 * (kWX / 16);
+    *reinterpret_cast<uint4 *>(smem + st * kWStage + 3 * 4 * kWX + e * 16) =
+        make_uint4(e < kWX / 16 ? 0x3f80u : 0u, 0u, 0u, 0u);
+  }
+  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
+  volatile int *stop = &s_stop;
+  auto brick = [&](int u, int &b, int &x0, int &y0, int &z0) {
+    x0 = (u % pl.tx) * kTX;
+    u /= pl.tx;
+    y0 = (u % pl.ty) * kTY;
+    u /= pl.ty;
+    z0 = u % g.D;
+    b = u / g.D;
+  };
+
+  bool ok = true;
+  if (warp < kLoadWarps) {
+    // ---- brick copies: thread t keeps the 8-channel piece t mod 4 and steps over voxels ----
+    constexpr int VS = kLoadWarps * 8, NVX = kPX * (kTY + 2), NX = (NVX + VS - 1) / VS, NG = kTX * kTY / VS;
+    const int q = tid & 3, v0 = tid >> 2;
+    const int cb = sl * 32;
+    const bool half = cb < a.c1;
+    const int hs = half ? 1 : 0, C = half ? a.c1 : a.c0, Hs = g.H >> hs, Ws = g.W >> hs, Ds = g.D >> hs;
+    const bf16 *xb = (half ? a.x1 + cb : a.x0 + (cb - a.c1)) + q * 8;
+    const bf16 *gb = a.g + nt * 32 + q * 8;
+    auto landed = [&](int st) {  // this warp's copies into stage st are visible to the tensor cores
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full(st));
+    };
+    int s = 0, prev = -1;
+    uint32_t ph = 1;
+    for (int u = first; u < pl.bricks; u += pl.per) {
+      int b, x0, y0, z0;
+      brick(u, b, x0, y0, z0);
+      ok = __all_sync(0xffffffffu, mbar_wait(empty(s), ph, stop));
+      if (!ok) break;
+      const uint32_t sx = base + kWStage * s + q * kWX, sg = base + kWStage * s + 4 * 4 * kWX + q * kWG;
+      int off[NX];
+#pragma unroll
+      for (int i = 0; i < NX; ++i) {
+        const int v = v0 + i * VS, vy = v / kPX, vx = v - vy * kPX, y = y0 + vy - 1, x = x0 + vx - 1;
+        off[i] = (unsigned)y < (unsigned)g.H && (unsigned)x < (unsigned)g.W ? ((y >> hs) * Ws + (x >> hs)) * C : -1;
+      }
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const int z = z0 + j - 1;
+        const bool inz = z >= 0 && z < g.D;
+        const bf16 *plane = xb + ((size_t)b * Ds + (inz ? z >> hs : 0)) * Hs * Ws * C;
+#pragma unroll
+        for (int i = 0; i < NX; ++i) {
+          const int v = v0 + i * VS;
+          if (v < NVX)
+            cp16(sx + j * 4 * kWX + v * 16, plane + max(off[i], 0), inz && off[i] >= 0 ? 16 : 0);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < NG; ++i) {
+        const int v = v0 + i * VS, y = y0 + v / kTX, x = x0 + v % kTX;
+        const bool in = y < g.H && x < g.W;
+        const size_t vox = (((size_t)b * g.D + z0) * g.H + (in ? y : 0)) * g.W + (in ? x : 0);
+        cp16(sg + v * 16, gb + vox * a.cout, in ? 16 : 0);
+      }
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+      if (prev >= 0) {  // the next brick's copies are issued before this one's are waited for
+        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        landed(prev);
+      }
+      prev = s;
+      if (++s == kWStages) {
+        s = 0;
+        ph ^= 1;
+      }
+    }
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    if (prev >= 0) landed(prev);
+  } else {
+    // ---- MMA issue ----
+    // F32 <- BF16 x BF16, A and B MN-major (bits 15, 16), N = 32, M = 128
+    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | (4u << 17) | (8u << 24);
+    // MN-major: the stride word is between 8-channel pieces, the leading word between 8-voxel groups of K
+    const uint32_t ahi = desc_hi(kWX), bhi = desc_hi(kWG);
+    const bool issue = elect_one();
+    int s = 0;
+    uint32_t ph = 0, add = 0;
+    for (int u = first; u < pl.bricks; u += pl.per) {
+      int b, x0, y0, z0;
+      brick(u, b, x0, y0, z0);
+      ok = __all_sync(0xffffffffu, mbar_wait(full(s), ph, stop));
+      if (!ok) break;
+      fence_after();
+      const int nk = min(kTY / 2, (g.H - y0 + 1) / 2);  // 16-voxel steps (two rows of y)
+      const uint32_t blo = uniform(desc_lo(base + kWStage * s + 4 * 4 * kWX, kTX * 16));
+      const uint32_t acc = uniform(add);
+      uint32_t tap = uniform(desc_lo(base + kWStage * s, kPX * 16)), d = tmem;
+#pragma unroll 1
+      for (int yx = 0; yx < 9; ++yx) {
+        if (issue) {
+#pragma unroll
+          for (int ks = 0; ks < kTY / 2; ++ks)
+            if (ks < nk) mma_f16(d, tap + ks * 2 * kPX, ahi, blo + ks * 2 * kTX, bhi, idesc, ks ? 1u : acc);
+        }
+        __syncwarp();
+        tap += yx % 3 == 2 ? kPX - 2 : 1;
+        d += 32;
+      }
+      add = 1;
+      if (issue) mma_commit(empty(s));
+      __syncwarp();
+      if (++s == kWStages) {
+        s = 0;
+        ph ^= 1;
+      }
+    }
+    if (issue) mma_commit(done);
+    __syncwarp();
+  }
+  if (warp < 4 || (!ok && warp == kLoadWarps)) {
+    // every MMA has finished (also after a failure, before TMEM is given back)
+    const unsigned long long t0 = now_ns();
+    bool fin = mbar_try(done, 0);
+    while (!fin && now_ns() - t0 < kWaitNs) fin = mbar_try(done, 0);
+    if (!fin) *stop = 1;
+    ok = __all_sync(0xffffffffu, fin && ok);
+  }
+  if (warp < 4 && ok && first < pl.bricks) {
+    fence_after();
+    const uint32_t rows = tmem + ((uint32_t)(warp * 32) << 16);
+    uint32_t v[32];
+    if (warp < 3) {  // warp w holds tap plane dz = w - 1, a lane one input channel of the slice
+      const int cin = a.c0 + a.c1;
+      float *dst = a.dw + (size_t)(nt * 32) * 27 * cin + (size_t)(warp * 9) * cin + sl * 32 + lane;
+      for (int yx = 0; yx < 9; ++yx) {
+        tmem_ld32(v, rows + yx * 32);
+#pragma unroll
+        for (int o = 0; o < 32; ++o) atomicAdd(dst + ((size_t)o * 27 + yx) * cin, __uint_as_float(v[o]));
+      }
+    } else if (sl == 0) {  // row 96: the sums of G
+      tmem_ld32(v, rows);
+      if (lane == 0)
+#pragma unroll
+        for (int o = 0; o < 32; ++o) atomicAdd(a.db + nt * 32 + o, __uint_as_float(v[o]));
+    }
+    fence_before();
+  }
+  __syncwarp();
+  fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTmemCols));
+  }
+  if (tid == 0 && *stop) *reinterpret_cast<volatile int *>(a.err) = 1;
+}
+
 // Tensor-core cycles of one plane that serves n output planes (per 16-channel
 // step, 128-voxel tile and (dy, dx)): the products at N / 2 cycles for M = 128,
 // K = 16, or the operands' 128-byte shared-memory reads, whichever is longer.
@@ -644,6 +863,25 @@ cudaError_t conv_prepare() {
   if (e == cudaSuccess) e = prepare<64, 128>();
   if (e == cudaSuccess) e = prepare<32, 64>();
   return e;
+}
+
+cudaError_t wgrad_prepare() {
+  return cudaFuncSetAttribute(wgrad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWStages * kWStage);
+}
+
+cudaError_t wgrad_launch(const WgradTcArgs &a, int num_sms, cudaStream_t stream) {
+  if (a.c0 % 32 || a.c1 % 32 || a.cout % 32) return cudaErrorInvalidValue;
+  WPlan pl;
+  pl.nsl = (a.c0 + a.c1) / 32;
+  pl.nt = a.cout / 32;
+  pl.tx = (a.vol.W + kTX - 1) / kTX;
+  pl.ty = (a.vol.H + kTY - 1) / kTY;
+  pl.bricks = a.vol.B * a.vol.D * pl.tx * pl.ty;
+  pl.per = num_sms / (pl.nsl * pl.nt);
+  if (pl.per < 1) pl.per = 1;
+  if (pl.per > pl.bricks) pl.per = pl.bricks;
+  wgrad_tc_kernel<<<pl.nsl * pl.nt * pl.per, kWThreads, kWStages * kWStage, stream>>>(a, pl);
+  return cudaGetLastError();
 }
 
 cudaError_t conv_launch(const ConvArgs &a, int num_sms, cudaStream_t stream) {

@@ -48,4 +48,19 @@ cudaError_t conv_prepare();
 // (128, 0), (64, 128), (32, 64); cout a multiple of 32.
 cudaError_t conv_launch(const ConvArgs &a, int num_sms, cudaStream_t stream);
 
+// dw[o][tap][c] += sum_p g[p][o] x[p + delta_tap][c] and db[o] += sum_p g[p][o], x the concatenation of x1
+// (through nearest upsampling, its channels first) and x0 as in ConvArgs; channel
+// counts multiples of 32.
+struct WgradTcArgs {
+  const bf16 *g;      // [V][cout]
+  const bf16 *x0, *x1;
+  float *dw;          // [cout][27][c1 + c0]
+  float *db;          // [cout]
+  int c0, c1, cout;
+  Vol vol;
+  int *err;
+};
+cudaError_t wgrad_prepare();
+cudaError_t wgrad_launch(const WgradTcArgs &a, int num_sms, cudaStream_t stream);
+
 }  // namespace s3ttv_net_detail
