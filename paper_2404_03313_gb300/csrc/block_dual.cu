@@ -1305,6 +1305,16 @@ constexpr int kSW = 4;         // warps per CTA
 constexpr int kCW = 32;        // columns per chunk (four 8-column k-steps)
 constexpr int kCS = kCW + 4;   // chunk row stride: 4 mod 32 words (conflict-free Gram fragments)
 
+// CTAs per SM.  A warp's block is a chain of dependent loads, products and shuffles,
+// so more warps help until their loads crowd the L1: k = 5 fills an SM's shared memory
+// with four CTAs, k = 3 is best with five, the others with six (80 registers).  The block
+// duals of a pass, exact / first-order steps, ms, with four CTAs -> now (and with 5, 6, 8):
+// 256x256x128: k = 1 .287/.290 -> .258/.258 (.263, .258, .262), k = 2 .407/.377 ->
+// .334/.305 (.340, .334, .348), k = 3 .756/.611 -> .727/.586 (.727, .746, .774), k = 4
+// 1.103/.838 -> 1.047/.793 (1.066, 1.047; seven 1.062); 97x131x61: k = 2 .065/.059 ->
+// .047/.042, k = 3 .124/.096 -> .109/.084, k = 4 .182/.132 -> .160/.114.
+__host__ __device__ constexpr int stream_ctas(int k) { return k == 5 ? 4 : (k == 3 ? 5 : 6); }
+
 template <int K>
 struct StreamLayout {
   static constexpr int n = K * K;
@@ -1621,7 +1631,7 @@ __device__ void stream_block(const BlockDualArgs &a, long long l, float *bufs, u
 }
 
 template <int K>
-__global__ void __launch_bounds__(kSW * 32, 4) block_dual_stream_kernel(BlockDualArgs a) {
+__global__ void __launch_bounds__(kSW * 32, stream_ctas(K)) block_dual_stream_kernel(BlockDualArgs a) {
   chained();
   extern __shared__ __align__(16) float smem[];
   if (a.sc->done) return;
@@ -1643,7 +1653,7 @@ __global__ void __launch_bounds__(kSW * 32, 4) block_dual_stream_kernel(BlockDua
 // items[i + 1].first)), taken by the warps of one persistent grid; each
 // problem keeps its own sizes, step size, stop flag and statistics.
 template <int K>
-__global__ void __launch_bounds__(kSW * 32, 4) block_dual_stream_batch_kernel(const BatchDual *items, int n,
+__global__ void __launch_bounds__(kSW * 32, stream_ctas(K)) block_dual_stream_batch_kernel(const BatchDual *items, int n,
                                                                               long long total) {
   chained();
   extern __shared__ __align__(16) float smem[];
