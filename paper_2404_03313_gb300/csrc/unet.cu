@@ -43,12 +43,15 @@
 
 #include <new>
 
+#include "chain.cuh"
 #include "s3ttv.h"
 #include "unet_conv.cuh"
 
 namespace {
 
 using namespace s3ttv_net_detail;
+using s3ttv::chained;
+using s3ttv::launch_chained;
 
 constexpr int kLayers = 10;
 constexpr int kCin[kLayers] = {1, 32, 32, 64, 64, 128, 192, 64, 96, 32};
@@ -162,6 +165,7 @@ constexpr int kFirstSmem = kStages * kWS * 2 * kAS * (int)sizeof(bf16);
 
 __global__ void __launch_bounds__(128) wgrad_first_kernel(const bf16 *G, const bf16 *N, float *dw, float *db, int V,
                                                           int chunk) {
+  chained();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   bf16 *Gs = reinterpret_cast<bf16 *>(smem_raw);
   bf16 *Xs = Gs + kStages * kWS * kAS;
@@ -225,6 +229,7 @@ __global__ void __launch_bounds__(128) wgrad_first_kernel(const bf16 *G, const b
 // this takes 374 us.  Every output sums its 27 taps in the same order.
 __global__ void __launch_bounds__(256, 2) conv_first_kernel(const float *v, const bf16 *w, const float *bias, bf16 *y,
                                                          Vol g) {
+  chained();
   __shared__ __align__(16) float ws[27][32];
   __shared__ __align__(16) float bs[32];
   for (int i = threadIdx.x; i < 32 * 27; i += blockDim.x) ws[i % 27][i / 27] = __bfloat162float(w[i]);
@@ -283,6 +288,7 @@ __global__ void __launch_bounds__(256, 2) conv_first_kernel(const float *v, cons
 // that column 27 of the weight gradient is the bias gradient) and four zeros: the first layer's input as 32 BF16 channels, so its weight
 // gradient runs on the tensor-core weight-gradient kernel.
 __global__ void __launch_bounds__(256) im2col_first_kernel(const float *v, bf16 *col, Vol g) {
+  chained();
   const int V = nvox(g);
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < V; p += gridDim.x * blockDim.x) {
     int b, z, y, x;
@@ -307,6 +313,7 @@ __global__ void __launch_bounds__(256) im2col_first_kernel(const float *v, bf16 
 // mode 1: y[q] = (sum of the 8 children of q in x[., coff : coff + C] (stride cx))
 //         zeroed where mask[q] <= 0 (transpose of nearest upsampling, then ReLU mask).
 __global__ void pool_kernel(const bf16 *x, int cx, int coff, const bf16 *mask, bf16 *y, int C, Vol lo, int mode) {
+  chained();
   const int pieces = C / 8;
   const long long n = (long long)nvox(lo) * pieces;
   const int Dh = 2 * lo.D, Hh = 2 * lo.H, Wh = 2 * lo.W;
@@ -340,6 +347,7 @@ __global__ void pool_kernel(const bf16 *x, int cx, int coff, const bf16 *mask, b
 // the gradient of a tensor that feeds both a pooling and a skip connection.
 __global__ void combine_kernel(const bf16 *glo, const bf16 *ghi, int chi, int coff, const bf16 *mask, bf16 *y, int C,
                                Vol hi) {
+  chained();
   const int pieces = C / 8;
   const long long n = (long long)nvox(hi) * pieces;
   const int Dl = hi.D / 2, Hl = hi.H / 2, Wl = hi.W / 2;
@@ -366,6 +374,7 @@ __global__ void combine_kernel(const bf16 *glo, const bf16 *ghi, int chi, int co
 __global__ void __launch_bounds__(256) head_bwd_kernel(const bf16 *f, const float *v, const float *hp,
                                                        const float *tu, const float *ts, const float *tt, int V,
                                                        float inv_n, bf16 *G, float *dwh, double *loss) {
+  chained();
   __shared__ float w[kHeadIn * kHeadOut + kHeadOut];
   __shared__ float red[8][kHeadIn * kHeadOut + kHeadOut];
   __shared__ double lred[8];
@@ -446,6 +455,7 @@ __global__ void __launch_bounds__(256) head_bwd_kernel(const bf16 *f, const floa
 // ---------------------------------------------------------------- optimiser and weight packing
 __global__ void adam_kernel(float *theta, const float *g, float *m, float *s, long long n, float lr, float b1,
                             float b2, float eps, float c1, float c2) {
+  chained();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const float gi = g[i];
     const float mi = fmaf(b1, m[i], (1.f - b1) * gi);
@@ -462,6 +472,7 @@ __global__ void adam_kernel(float *theta, const float *g, float *m, float *s, lo
 // is w[o][tap][c] (wb); hp = the head with its weights rounded to BF16 and its
 // bias in FP32.
 __global__ void pack_kernel(const float *theta, LayerTable t, bf16 *wf, bf16 *wb, float *hp) {
+  chained();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < t.total; i += (long long)gridDim.x * blockDim.x) {
     const float x = theta[i];
     if (i >= t.hw_off) {
@@ -656,17 +667,15 @@ const float *bias(const s3ttv_net *net, int l) { return net->theta + net->tab.bo
 int run_forward(s3ttv_net *net, const float *v, const Vol &g0, float *const *out = nullptr) {
   const Vol g1 = half(g0), g2 = half(g1);
   const int V0 = nvox(g0), V1 = nvox(g1), V2 = nvox(g2);
-  conv_first_kernel<<<grid_for(net, V0, 256), 256, 0, net->stream>>>(v, wf(net, 0), bias(net, 0), net->e1a, g0);
-  NCU(cudaGetLastError());
+  NCU(launch_chained(conv_first_kernel, grid_for(net, V0, 256), 256, 0, net->stream, v, wf(net, 0), bias(net, 0),
+                     net->e1a, g0));
   NCU(launch_conv(net, net->e1a, 32, nullptr, 0, wf(net, 1), bias(net, 1), nullptr, net->e1b, 32, true, g0));
-  pool_kernel<<<grid_for(net, (long long)V1 * 4, 256), 256, 0, net->stream>>>(net->e1b, 32, 0, nullptr, net->p1, 32,
-                                                                               g1, 0);
-  NCU(cudaGetLastError());
+  NCU(launch_chained(pool_kernel, grid_for(net, (long long)V1 * 4, 256), 256, 0, net->stream, net->e1b, 32, 0,
+                     nullptr, net->p1, 32, g1, 0));
   NCU(launch_conv(net, net->p1, 32, nullptr, 0, wf(net, 2), bias(net, 2), nullptr, net->e2a, 64, true, g1));
   NCU(launch_conv(net, net->e2a, 64, nullptr, 0, wf(net, 3), bias(net, 3), nullptr, net->e2b, 64, true, g1));
-  pool_kernel<<<grid_for(net, (long long)V2 * 8, 256), 256, 0, net->stream>>>(net->e2b, 64, 0, nullptr, net->p2, 64,
-                                                                               g2, 0);
-  NCU(cudaGetLastError());
+  NCU(launch_chained(pool_kernel, grid_for(net, (long long)V2 * 8, 256), 256, 0, net->stream, net->e2b, 64, 0,
+                     nullptr, net->p2, 64, g2, 0));
   NCU(launch_conv(net, net->p2, 64, nullptr, 0, wf(net, 4), bias(net, 4), nullptr, net->ba, 128, true, g2));
   NCU(launch_conv(net, net->ba, 128, nullptr, 0, wf(net, 5), bias(net, 5), nullptr, net->bb, 128, true, g2));
   NCU(launch_conv(net, net->e2b, 64, net->bb, 128, wf(net, 6), bias(net, 6), nullptr, net->d2a, 64, true, g1));
@@ -694,9 +703,8 @@ int run_backward(s3ttv_net *net, const float *v, const float *tu, const float *t
   NCU(cudaMemsetAsync(G, 0, sizeof(float) * T.total, net->stream));
   NCU(cudaMemsetAsync(net->loss, 0, sizeof(double), net->stream));
   const float inv_n = (float)(1.0 / (3.0 * (double)V0));
-  head_bwd_kernel<<<grid_for(net, V0, 256), 256, 0, net->stream>>>(net->d1b, v, net->hp, tu, ts, tt, V0, inv_n,
-                                                                   net->gB0, G + T.hw_off, net->loss);
-  NCU(cudaGetLastError());
+  NCU(launch_chained(head_bwd_kernel, grid_for(net, V0, 256), 256, 0, net->stream, net->d1b, v, net->hp, tu, ts, tt,
+                     V0, inv_n, net->gB0, G + T.hw_off, net->loss));
   auto wgrad = [&](int l, const bf16 *gout, const bf16 *x0, int c0, const bf16 *x1, int c1, const Vol &g) {
     return launch_wgrad(net, gout, T.cout[l], x0, c0, x1, c1, G + T.woff[l], G + T.boff[l], g);
   };
@@ -706,18 +714,16 @@ int run_backward(s3ttv_net *net, const float *v, const float *tu, const float *t
   // d1a: gC0 -> gA0 [up(d2b) 64 | e1b 32]
   NCU(wgrad(8, net->gC0, net->e1b, 32, net->d2b, 64, g0));
   NCU(launch_conv(net, net->gC0, 32, nullptr, 0, wbk(net, 8), nullptr, nullptr, net->gA0, 96, false, g0));
-  pool_kernel<<<grid_for(net, (long long)V1 * 8, 256), 256, 0, net->stream>>>(net->gA0, 96, 0, net->d2b, net->gB1,
-                                                                               64, g1, 1);
-  NCU(cudaGetLastError());
+  NCU(launch_chained(pool_kernel, grid_for(net, (long long)V1 * 8, 256), 256, 0, net->stream, net->gA0, 96, 0,
+                     net->d2b, net->gB1, 64, g1, 1));
   // d2b: gB1 -> gC1 (masked by d2a)
   NCU(wgrad(7, net->gB1, net->d2a, 64, nullptr, 0, g1));
   NCU(launch_conv(net, net->gB1, 64, nullptr, 0, wbk(net, 7), nullptr, net->d2a, net->gC1, 64, false, g1));
   // d2a: gC1 -> gA1 [up(bb) 128 | e2b 64]
   NCU(wgrad(6, net->gC1, net->e2b, 64, net->bb, 128, g1));
   NCU(launch_conv(net, net->gC1, 64, nullptr, 0, wbk(net, 6), nullptr, nullptr, net->gA1, 192, false, g1));
-  pool_kernel<<<grid_for(net, (long long)V2 * 16, 256), 256, 0, net->stream>>>(net->gA1, 192, 0, net->bb, net->gB2,
-                                                                                128, g2, 1);
-  NCU(cudaGetLastError());
+  NCU(launch_chained(pool_kernel, grid_for(net, (long long)V2 * 16, 256), 256, 0, net->stream, net->gA1, 192, 0,
+                     net->bb, net->gB2, 128, g2, 1));
   // bb: gB2 -> gC2 (masked by ba)
   NCU(wgrad(5, net->gB2, net->ba, 128, nullptr, 0, g2));
   NCU(launch_conv(net, net->gB2, 128, nullptr, 0, wbk(net, 5), nullptr, net->ba, net->gC2, 128, false, g2));
@@ -725,38 +731,33 @@ int run_backward(s3ttv_net *net, const float *v, const float *tu, const float *t
   NCU(wgrad(4, net->gC2, net->p2, 64, nullptr, 0, g2));
   NCU(launch_conv(net, net->gC2, 128, nullptr, 0, wbk(net, 4), nullptr, nullptr, net->gB2, 64, false, g2));
   // e2b: pool transpose + skip part of gA1, masked by e2b -> gB1
-  combine_kernel<<<grid_for(net, (long long)V1 * 8, 256), 256, 0, net->stream>>>(net->gB2, net->gA1, 192, 128,
-                                                                                  net->e2b, net->gB1, 64, g1);
-  NCU(cudaGetLastError());
+  NCU(launch_chained(combine_kernel, grid_for(net, (long long)V1 * 8, 256), 256, 0, net->stream, net->gB2, net->gA1,
+                     192, 128, net->e2b, net->gB1, 64, g1));
   NCU(wgrad(3, net->gB1, net->e2a, 64, nullptr, 0, g1));
   NCU(launch_conv(net, net->gB1, 64, nullptr, 0, wbk(net, 3), nullptr, net->e2a, net->gC1, 64, false, g1));
   // e2a: gC1 -> gradient of p1 (32 channels, into gB1)
   NCU(wgrad(2, net->gC1, net->p1, 32, nullptr, 0, g1));
   NCU(launch_conv(net, net->gC1, 64, nullptr, 0, wbk(net, 2), nullptr, nullptr, net->gB1, 32, false, g1));
   // e1b: pool transpose + skip part of gA0, masked by e1b -> gB0
-  combine_kernel<<<grid_for(net, (long long)V0 * 4, 256), 256, 0, net->stream>>>(net->gB1, net->gA0, 96, 64,
-                                                                                  net->e1b, net->gB0, 32, g0);
-  NCU(cudaGetLastError());
+  NCU(launch_chained(combine_kernel, grid_for(net, (long long)V0 * 4, 256), 256, 0, net->stream, net->gB1, net->gA0,
+                     96, 64, net->e1b, net->gB0, 32, g0));
   NCU(wgrad(1, net->gB0, net->e1a, 32, nullptr, 0, g0));
   NCU(launch_conv(net, net->gB0, 32, nullptr, 0, wbk(net, 1), nullptr, net->e1a, net->gC0, 32, false, g0));
   // e1a (one input channel): its 27 neighbour values as 32 channels (into gA0,
   // free by now), then the weight gradient of one unshifted tap
-  im2col_first_kernel<<<grid_for(net, V0, 256), 256, 0, net->stream>>>(v, net->gA0, g0);
-  NCU(cudaGetLastError());
+  NCU(launch_chained(im2col_first_kernel, grid_for(net, V0, 256), 256, 0, net->stream, v, net->gA0, g0));
   {
     const int ctas = net->num_sms * 2;
     const int chunk = ((V0 + ctas - 1) / ctas + kWS - 1) / kWS * kWS;
-    wgrad_first_kernel<<<(V0 + chunk - 1) / chunk, 128, kFirstSmem, net->stream>>>(net->gC0, net->gA0, G + T.woff[0],
-                                                                                   G + T.boff[0], V0, chunk);
-    NCU(cudaGetLastError());
+    NCU(launch_chained(wgrad_first_kernel, (V0 + chunk - 1) / chunk, 128, kFirstSmem, net->stream, net->gC0, net->gA0,
+                       G + T.woff[0], G + T.boff[0], V0, chunk));
   }
   return S3TTV_OK;
 }
 
 int pack(s3ttv_net *net) {
-  pack_kernel<<<grid_for(net, net->tab.total, 256), 256, 0, net->stream>>>(net->theta, net->tab, net->wf, net->wb,
-                                                                           net->hp);
-  NCU(cudaGetLastError());
+  NCU(launch_chained(pack_kernel, grid_for(net, net->tab.total, 256), 256, 0, net->stream, net->theta, net->tab,
+                     net->wf, net->wb, net->hp));
   return S3TTV_OK;
 }
 
@@ -921,9 +922,8 @@ int s3ttv_net_train_step(s3ttv_net *net, const float *v, const float *u_ref, con
   const double b1 = 0.9, b2 = 0.999;
   const float c1 = (float)(1.0 / (1.0 - pow(b1, (double)net->adam_t)));
   const float c2 = (float)(1.0 / (1.0 - pow(b2, (double)net->adam_t)));
-  adam_kernel<<<grid_for(net, net->tab.total, 256), 256, 0, net->stream>>>(
-      net->theta, net->grad, net->m1, net->m2, net->tab.total, lr, (float)b1, (float)b2, 1e-8f, c1, c2);
-  NCU(cudaGetLastError());
+  NCU(launch_chained(adam_kernel, grid_for(net, net->tab.total, 256), 256, 0, net->stream, net->theta, net->grad,
+                     net->m1, net->m2, net->tab.total, lr, (float)b1, (float)b2, 1e-8f, c1, c2));
   if ((rc = pack(net))) return rc;
   return finish(net);
 }

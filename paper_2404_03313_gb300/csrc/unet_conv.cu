@@ -30,9 +30,13 @@
 // sets the error flag and ends.
 #include "unet_conv.cuh"
 
+#include "chain.cuh"
+
 #include <stdint.h>
 
 namespace s3ttv_net_detail {
+using s3ttv::chained;
+using s3ttv::launch_chained;
 namespace {
 
 constexpr int kEpiWarps = 8, kMmaWarp = 8, kWWarp = 10, kLoadWarp0 = 11, kLoadWarps = 8;
@@ -188,6 +192,7 @@ __device__ __forceinline__ Unit unit_at(int u, const Plan &pl, const Vol &g) {
 
 template <int C0, int C1, int J>
 __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan pl) {
+  chained();
   constexpr int CIN = C0 + C1, NQ = CIN / 8;
   constexpr int CS = stage_channels(CIN), NS = CIN / CS;  // channels per weight stage
   constexpr bool RES = weights_resident(CIN);
@@ -577,6 +582,7 @@ struct WPlan {
 };
 
 __global__ void __launch_bounds__(kWThreads, 1) wgrad_tc_kernel(WgradTcArgs a, WPlan pl) {
+  chained();
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) uint64_t bars[2 * kWStages + 1];
   __shared__ uint32_t s_tmem;
@@ -839,11 +845,8 @@ bool make_plan(const ConvArgs &a, int num_sms, Plan *best) {
 template <int C0, int C1>
 cudaError_t launch(const ConvArgs &a, const Plan &pl, int num_sms, cudaStream_t stream) {
   const int ctas = num_sms > pl.nn ? num_sms / pl.nn : 1, grid = pl.nn * (pl.units < ctas ? pl.units : ctas);
-  if (pl.J == 2)
-    conv_tc_kernel<C0, C1, 2><<<grid, kThreads, pl.smem, stream>>>(a, pl);
-  else
-    conv_tc_kernel<C0, C1, 1><<<grid, kThreads, pl.smem, stream>>>(a, pl);
-  return cudaGetLastError();
+  return launch_chained(pl.J == 2 ? conv_tc_kernel<C0, C1, 2> : conv_tc_kernel<C0, C1, 1>, grid, kThreads, pl.smem,
+                        stream, a, pl);
 }
 
 template <int C0, int C1>
@@ -880,8 +883,7 @@ cudaError_t wgrad_launch(const WgradTcArgs &a, int num_sms, cudaStream_t stream)
   pl.per = num_sms / (pl.nsl * pl.nt);
   if (pl.per < 1) pl.per = 1;
   if (pl.per > pl.bricks) pl.per = pl.bricks;
-  wgrad_tc_kernel<<<pl.nsl * pl.nt * pl.per, kWThreads, kWStages * kWStage, stream>>>(a, pl);
-  return cudaGetLastError();
+  return launch_chained(wgrad_tc_kernel, pl.nsl * pl.nt * pl.per, kWThreads, kWStages * kWStage, stream, a, pl);
 }
 
 cudaError_t conv_launch(const ConvArgs &a, int num_sms, cudaStream_t stream) {
