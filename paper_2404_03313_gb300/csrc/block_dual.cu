@@ -542,7 +542,10 @@ __device__ void form_M(float *Gm) {
 // TF32 products per FP32 product): rows [0, MR) of A, columns [0, NC) of B and
 // the inner index [0, KD) are read through the accessors, everything else is
 // zero.  d[m][q][e] is element (16 m + g + 8 (e >> 1), 8 q + 2 t + (e & 1)) of
-// the 32 x 32 result (g = lane / 4, t = lane % 4).
+// the 32 x 32 result (g = lane / 4, t = lane % 4).  For 25 rows (k = 5) the loop over
+// the inner index stays rolled: its copies, unrolled, are most of a kernel whose 16
+// warps an SM wait for instructions (block duals of a 256 x 256 x 128 pass, exact /
+// first-order steps: 2.40 / 1.68 ms unrolled, 2.35 / 1.65 rolled).
 template <int MR, int NC, int KD, class FA, class FB>
 __device__ __forceinline__ void mm32(const FA &A, const FB &B, float (&d)[2][4][4]) {
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -550,7 +553,7 @@ __device__ __forceinline__ void mm32(const FA &A, const FB &B, float (&d)[2][4][
   for (int m = 0; m < 2; ++m)
 #pragma unroll
     for (int q = 0; q < 4; ++q) d[m][q][0] = d[m][q][1] = d[m][q][2] = d[m][q][3] = 0.f;
-#pragma unroll
+#pragma unroll(KD > 16 ? 1 : 4)
   for (int kk = 0; kk < (KD + 7) / 8; ++kk) {
     unsigned bh[4][2], bl[4][2];
 #pragma unroll
@@ -1305,14 +1308,20 @@ constexpr int kSW = 4;         // warps per CTA
 constexpr int kCW = 32;        // columns per chunk (four 8-column k-steps)
 constexpr int kCS = kCW + 4;   // chunk row stride: 4 mod 32 words (conflict-free Gram fragments)
 
-// CTAs per SM.  A warp's block is a chain of dependent loads, products and shuffles,
-// so more warps help until their loads crowd the L1: k = 5 fills an SM's shared memory
-// with four CTAs, k = 3 is best with five, the others with six (80 registers).  The block
-// duals of a pass, exact / first-order steps, ms, with four CTAs -> now (and with 5, 6, 8):
-// 256x256x128: k = 1 .287/.290 -> .258/.258 (.263, .258, .262), k = 2 .407/.377 ->
-// .334/.305 (.340, .334, .348), k = 3 .756/.611 -> .727/.586 (.727, .746, .774), k = 4
-// 1.103/.838 -> 1.047/.793 (1.066, 1.047; seven 1.062); 97x131x61: k = 2 .065/.059 ->
-// .047/.042, k = 3 .124/.096 -> .109/.084, k = 4 .182/.132 -> .160/.114.
+// Whole chunks take a copy of the chunk code without the ragged one's predicates, for
+// k <= 4 unrolled over the chunk so that its loads run ahead of the products.  k = 5
+// stays rolled: its kernel already waits for instructions (unrolled 2.49 / 1.92 ms a
+// pass instead of 2.34 / 1.64, see below).
+//
+// CTAs per SM.  A warp's block is a chain of dependent loads, products and shuffles
+// (no memory wait is left: a scheduler issues in 55 % of its cycles and waits mostly
+// for fixed latencies), so more warps help until their code and rows crowd the caches:
+// k = 5 is best with four CTAs (five: 2.40 / 1.71 ms), k = 3 with five, the others with
+// six.  The block duals of a pass, exact / first-order steps, ms, before (all with
+// four, no copy for whole chunks) -> now:
+// 256x256x128: k = 1 .287/.290 -> .225/.225, k = 2 .407/.377 -> .301/.274, k = 3 .756/.611
+// -> .683/.547, k = 4 1.103/.838 -> 1.025/.782, k = 5 2.42/1.70 -> 2.34/1.64;
+// 97x131x61: k = 4 .182/.132 -> .158/.113, k = 5 .403/.265 -> .385/.251.
 __host__ __device__ constexpr int stream_ctas(int k) { return k == 5 ? 4 : (k == 3 ? 5 : 6); }
 
 template <int K>
@@ -1320,9 +1329,9 @@ struct StreamLayout {
   static constexpr int n = K * K;
   static constexpr int buf = n * kCS;                          // one chunk buffer
   static constexpr int gm = gm_floats<K, true>();              // G, then M (by rows, stride GS)
-  static constexpr int off = 2 * buf + gm;                     // the rows' pixel offsets (n ints)
-  static constexpr int fb = (off + n + 3) & ~3;                // the chunk's F rows (n x kCW), step A
-  static constexpr int per_warp = fb + n * kCW;
+  static constexpr int fb = 2 * buf;                           // the chunk's F rows (n x kCW) in step A, over G's slot
+  static constexpr int off = 2 * buf + (gm > n * kCW ? gm : n * kCW);  // the rows' pixel offsets (n ints)
+  static constexpr int per_warp = (off + n + 3) & ~3;
   static_assert(w_floats<K>() + fo_floats<K>() <= 2 * buf, "W and the first-order scratch fit the chunk buffers");
 };
 
@@ -1408,52 +1417,58 @@ __device__ void stream_block(const BlockDualArgs &a, long long l, float *bufs, u
         cp_async_wait<0>();
       }
       __syncwarp();
-      const int c0 = ch * kCW, w4 = min(kCW, RW - c0) >> 2;
+      const int c0 = ch * kCW;
+      auto use = [&](auto full) {
+        const int w4 = full.value ? kCW / 4 : (RW - c0) >> 2;
 #pragma unroll
-      for (int u = 0; u < NE; ++u) {
-        const int e = lane + 32 * u, r = e >> 3, j = e & 7;
-        if (r < n && j < w4) {
-          float *dst = cur + r * kCS + 4 * j;
-          const float4 f = lds4(fb + r * kCW + 4 * j);
-          float4 y = lds4(dst);
-          y.x = fmaf(gY, f.x, y.x);
-          y.y = fmaf(gY, f.y, y.y);
-          y.z = fmaf(gY, f.z, y.z);
-          y.w = fmaf(gY, f.w, y.w);
-          sts4(dst, y);
-          // Y' replaces Y_l in global memory (kept in L2) for step C
-          st_hint(reinterpret_cast<float4 *>(Yl + (size_t)r * RW + c0) + j, y, pol_keep);
-        }
-      }
-      __syncwarp();  // every lane has read fb: the next chunk's F may replace it
-      if (ch + 1 < NCH) load_f(ch + 1);
-      const int nks = w4 >> 1;
-      for (int ks = 0; ks < nks; ++ks) {
-        unsigned xh[4][2], xl[4][2];
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            xh[q][h] = xl[q][h] = 0u;
-            if (8 * q < n) {
-              const int row = 8 * q + g;
-              split_tf32(row < n ? cur[row * kCS + 8 * ks + t + 4 * h] : 0.f, xh[q][h], xl[q][h]);
-            }
+        for (int u = 0; u < NE; ++u) {
+          const int e = lane + 32 * u, r = e >> 3, j = e & 7;
+          if (r < n && j < w4) {
+            float *dst = cur + r * kCS + 4 * j;
+            const float4 f = lds4(fb + r * kCW + 4 * j);
+            float4 y = lds4(dst);
+            y.x = fmaf(gY, f.x, y.x);
+            y.y = fmaf(gY, f.y, y.y);
+            y.z = fmaf(gY, f.z, y.z);
+            y.w = fmaf(gY, f.w, y.w);
+            sts4(dst, y);
+            // Y' replaces Y_l in global memory (kept in L2) for step C
+            st_hint(reinterpret_cast<float4 *>(Yl + (size_t)r * RW + c0) + j, y, pol_keep);
           }
-        const unsigned ah[2][4] = {{xh[0][0], xh[1][0], xh[0][1], xh[1][1]}, {xh[2][0], xh[3][0], xh[2][1], xh[3][1]}};
-        const unsigned al[2][4] = {{xl[0][0], xl[1][0], xl[0][1], xl[1][1]}, {xl[2][0], xl[3][0], xl[2][1], xl[3][1]}};
-        three_parts([&](auto P) {
-          int idx = 0;
+        }
+        __syncwarp();  // every lane has read fb: the next chunk's F may replace it
+        if (ch + 1 < NCH) load_f(ch + 1);
+        const int nks = w4 >> 1;
+#pragma unroll(K < 5 ? 4 : 1)
+        for (int ks = 0; ks < nks; ++ks) {
+          unsigned xh[4][2], xl[4][2];
 #pragma unroll
-          for (int m = 0; m < 2; ++m)
+          for (int q = 0; q < 4; ++q)
 #pragma unroll
-            for (int q = 0; q < 4; ++q)
-              if (T::need(m, q)) {
-                mma_3xtf32_part<decltype(P)::value>(acc[idx], ah[m], al[m], xh[q][0], xh[q][1], xl[q][0], xl[q][1]);
-                ++idx;
+            for (int h = 0; h < 2; ++h) {
+              xh[q][h] = xl[q][h] = 0u;
+              if (8 * q < n) {
+                const int row = 8 * q + g;
+                split_tf32(row < n ? cur[row * kCS + 8 * ks + t + 4 * h] : 0.f, xh[q][h], xl[q][h]);
               }
-        });
-      }
+            }
+          const unsigned ah[2][4] = {{xh[0][0], xh[1][0], xh[0][1], xh[1][1]}, {xh[2][0], xh[3][0], xh[2][1], xh[3][1]}};
+          const unsigned al[2][4] = {{xl[0][0], xl[1][0], xl[0][1], xl[1][1]}, {xl[2][0], xl[3][0], xl[2][1], xl[3][1]}};
+          three_parts([&](auto P) {
+            int idx = 0;
+#pragma unroll
+            for (int m = 0; m < 2; ++m)
+#pragma unroll
+              for (int q = 0; q < 4; ++q)
+                if (T::need(m, q)) {
+                  mma_3xtf32_part<decltype(P)::value>(acc[idx], ah[m], al[m], xh[q][0], xh[q][1], xl[q][0], xl[q][1]);
+                  ++idx;
+                }
+          });
+        }
+      };
+      if (RW - c0 >= kCW) use(std::true_type());
+      else use(std::false_type());
       __syncwarp();  // every lane has read this buffer before it is refilled
     }
     {  // G, both triangles, from the tiles reaching the upper triangle
@@ -1554,77 +1569,83 @@ __device__ void stream_block(const BlockDualArgs &a, long long l, float *bufs, u
         cp_async_wait<0>();
       }
       __syncwarp();
-      const int c0 = ch * kCW, w4 = min(kCW, RW - c0) >> 2, ntl = w4 >> 1;
-      // n-tiles of 8 columns, two at a time
-      for (int q = 0; q < ntl; q += 2) {
-        const bool two = q + 1 < ntl;
-        float d[2][NM][4];
+      const int c0 = ch * kCW;
+      auto use = [&](auto full) {
+        const int w4 = full.value ? kCW / 4 : (RW - c0) >> 2, ntl = w4 >> 1;
+        // n-tiles of 8 columns, two at a time
+#pragma unroll(K < 5 ? 2 : 1)
+        for (int q = 0; q < ntl; q += 2) {
+          const bool two = full.value || q + 1 < ntl;
+          float d[2][NM][4];
 #pragma unroll
-        for (int u = 0; u < 2; ++u)
+          for (int u = 0; u < 2; ++u)
 #pragma unroll
-          for (int m = 0; m < NM; ++m) d[u][m][0] = d[u][m][1] = d[u][m][2] = d[u][m][3] = 0.f;
+            for (int m = 0; m < NM; ++m) d[u][m][0] = d[u][m][1] = d[u][m][2] = d[u][m][3] = 0.f;
 #pragma unroll
-        for (int kk = 0; kk < NKS; ++kk) {
-          const int s0 = 8 * kk + t, s1 = s0 + 4;
-          unsigned bh[2][2], bl[2][2];
+          for (int kk = 0; kk < NKS; ++kk) {
+            const int s0 = 8 * kk + t, s1 = s0 + 4;
+            unsigned bh[2][2], bl[2][2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+              const float *col = cur + 8 * (q + u) + g;
+              const bool in = u == 0 || two;
+              split_tf32(in && s0 < S0 ? col[s0 * kCS] : 0.f, bh[u][0], bl[u][0]);
+              split_tf32(in && s1 < S0 ? col[s1 * kCS] : 0.f, bh[u][1], bl[u][1]);
+            }
+            three_parts([&](auto P) {
+#pragma unroll
+              for (int m = 0; m < NM; ++m)
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                  mma_3xtf32_part<decltype(P)::value>(d[u][m], mh[m][kk], ml[m][kk], bh[u][0], bh[u][1], bl[u][0],
+                                                      bl[u][1]);
+            });
+          }
 #pragma unroll
           for (int u = 0; u < 2; ++u) {
-            const float *col = cur + 8 * (q + u) + g;
-            const bool in = u == 0 || two;
-            split_tf32(in && s0 < S0 ? col[s0 * kCS] : 0.f, bh[u][0], bl[u][0]);
-            split_tf32(in && s1 < S0 ? col[s1 * kCS] : 0.f, bh[u][1], bl[u][1]);
+            if (u == 1 && !two) break;
+            const int c = 8 * (q + u) + 2 * t;
+#pragma unroll
+            for (int j = 0; j < NR; ++j) {
+              const float2 y = *reinterpret_cast<const float2 *>(cur + (S0 + j) * kCS + c);
+#pragma unroll
+              for (int m = 0; m < NM; ++m)
+#pragma unroll
+                for (int e2 = 0; e2 < 2; ++e2) {
+                  d[u][m][2 * e2] = fmaf(mr[m][e2][j], y.x, d[u][m][2 * e2]);
+                  d[u][m][2 * e2 + 1] = fmaf(mr[m][e2][j], y.y, d[u][m][2 * e2 + 1]);
+                }
+            }
           }
-          three_parts([&](auto P) {
+          __syncwarp();  // every lane has read these columns
 #pragma unroll
-            for (int m = 0; m < NM; ++m)
-#pragma unroll
-              for (int u = 0; u < 2; ++u)
-                mma_3xtf32_part<decltype(P)::value>(d[u][m], mh[m][kk], ml[m][kk], bh[u][0], bh[u][1], bl[u][0],
-                                                    bl[u][1]);
-          });
-        }
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          if (u == 1 && !two) break;
-          const int c = 8 * (q + u) + 2 * t;
-#pragma unroll
-          for (int j = 0; j < NR; ++j) {
-            const float2 y = *reinterpret_cast<const float2 *>(cur + (S0 + j) * kCS + c);
+          for (int u = 0; u < 2; ++u) {
+            if (u == 1 && !two) break;
+            const int c = 8 * (q + u) + 2 * t;
 #pragma unroll
             for (int m = 0; m < NM; ++m)
 #pragma unroll
               for (int e2 = 0; e2 < 2; ++e2) {
-                d[u][m][2 * e2] = fmaf(mr[m][e2][j], y.x, d[u][m][2 * e2]);
-                d[u][m][2 * e2 + 1] = fmaf(mr[m][e2][j], y.y, d[u][m][2 * e2 + 1]);
+                const int r = 16 * m + g + 8 * e2;
+                if (r < n) *reinterpret_cast<float2 *>(cur + r * kCS + c) = make_float2(d[u][m][2 * e2], d[u][m][2 * e2 + 1]);
               }
           }
         }
-        __syncwarp();  // every lane has read these columns
+        __syncwarp();  // Y_l of this chunk complete in the buffer
 #pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          if (u == 1 && !two) break;
-          const int c = 8 * (q + u) + 2 * t;
-#pragma unroll
-          for (int m = 0; m < NM; ++m)
-#pragma unroll
-            for (int e2 = 0; e2 < 2; ++e2) {
-              const int r = 16 * m + g + 8 * e2;
-              if (r < n) *reinterpret_cast<float2 *>(cur + r * kCS + c) = make_float2(d[u][m][2 * e2], d[u][m][2 * e2 + 1]);
-            }
+        for (int u = 0; u < NE; ++u) {
+          const int e = lane + 32 * u, r = e >> 3, j = e & 7;
+          if (r < n && j < w4) {
+            const int c = c0 + 4 * j;
+            const float4 y = lds4(cur + r * kCS + 4 * j);
+            __stcs(reinterpret_cast<float4 *>(Yl + (size_t)r * RW + c0) + j, y);
+            const bool hz = c >= N3p;
+            atomicAdd(reinterpret_cast<float4 *>((hz ? a.Zh : a.Zv) + (size_t)off[r] * N3p + (hz ? c - N3p : c)), y);
+          }
         }
-      }
-      __syncwarp();  // Y_l of this chunk complete in the buffer
-#pragma unroll
-      for (int u = 0; u < NE; ++u) {
-        const int e = lane + 32 * u, r = e >> 3, j = e & 7;
-        if (r < n && j < w4) {
-          const int c = c0 + 4 * j;
-          const float4 y = lds4(cur + r * kCS + 4 * j);
-          __stcs(reinterpret_cast<float4 *>(Yl + (size_t)r * RW + c0) + j, y);
-          const bool hz = c >= N3p;
-          atomicAdd(reinterpret_cast<float4 *>((hz ? a.Zh : a.Zv) + (size_t)off[r] * N3p + (hz ? c - N3p : c)), y);
-        }
-      }
+      };
+      if (RW - c0 >= kCW) use(std::true_type());
+      else use(std::false_type());
       __syncwarp();  // every lane has read this buffer before it is refilled
     }
   }
