@@ -893,7 +893,7 @@ def run_warm_start(args):
             "train_seconds": t_train, "targets_seconds": t_targets, "final_train_loss": losses[-1],
             "roofline": {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                          "frac": achieved / peak, "traffic": None,
-                         "kernel": "network forward (conv_fwd_kernel launches and the CUDA-core layers)",
+                         "kernel": "network forward (conv_tc_kernel launches and the CUDA-core first layer)",
                          "peak_source": "MEASURED_PEAKS.json bf16_tflops" if "bf16_tflops" in peaks
                          else "fallback 1900 TFLOP/s",
                          "flops_per_forward": flops, "forward_ms": fwd_ms},

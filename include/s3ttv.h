@@ -140,7 +140,7 @@ enum {
                                       context stays usable (host-side fault injection)    */
   S3TTV_OPT_NVTX = 15,             /* 1: NVTX ranges around each API call and each kernel
                                       class as a pass is enqueued (primal, l1-ball
-                                      thresholds, block dual, dual), for          
+                                      thresholds, block dual, dual), for
                                       profilers; 0 (default): none                        */
   S3TTV_OPT_JACOBI_POLISH_TOL = 16, /* relative orthogonality below which a pair of rows
                                       of the block eigen-solve is left as it is (0 <
