@@ -84,7 +84,6 @@ struct s3ttv_ctx {
 
 namespace {
 
-constexpr int kMaxGrid = 4096;
 constexpr int kMaxK = kMaxLargeK;  // k <= 5: block_dual.cu; 6..16: block_dual_large.cu
 // kernels enqueue_pass launches (without the re-solve): primal, l1 level 2 (with D D_s ubar
 // for the block-dual regularisers), l1 level 3, the regulariser's dual, dual
@@ -161,14 +160,9 @@ bool is_ssst(const s3ttv_ctx *c) { return c->reg == S3TTV_REG_SSST; }
 // parts of a block row: [D_v | D_h] (S3TTV, STV) or SSST's [D_v | D_h | D_s]
 int row_parts(const s3ttv_ctx *c) { return is_ssst(c) ? 3 : 2; }
 
-// CTAs of the elementwise kernels (512 threads, float4 pieces): at most two per SM.
 int elementwise_grid(const s3ttv_ctx *c, long long n) {
-  long long g = (n + 2047) / 2048;
-  long long cap = (long long)c->num_sms * 2;
-  if (cap > kMaxGrid) cap = kMaxGrid;
-  if (g > cap) g = cap;
-  if (g < 2) g = 2;
-  return (int)g;
+  const int g = elementwise_ctas(n, c->num_sms);
+  return g < 2 ? 2 : g;
 }
 
 void free_all(s3ttv_ctx *c) {

@@ -172,7 +172,7 @@ __device__ __forceinline__ void l1_scan_level(const L1Args &a, int pb) {
 // Shared memory adds integers natively but floats by compare-and-swap, and
 // neighbouring values crowd a few bins: with float sums the primal step took 109 us
 // at 256 x 256 x 128 once both projections were active, with these 67.  (The sums
-// stay below 2^32 up to 4 M elements per CTA, 1.2e9 per cube.)
+// stay below 2^32 up to 4 M elements per CTA: elementwise_ctas().)
 struct BinSums {
   unsigned cnt[kHistBins], hi[kHistBins], lo[kHistBins];
 };

@@ -99,11 +99,9 @@ extern "C" int s3ttv_l1_ball_static(const float *x, float *out, long long n, dou
   la.hsum = hsum;
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  long long grid = (n + 2047) / 2048;
-  const long long cap = (sms > 0 ? sms : 1) * 2ll;
-  if (grid > cap) grid = cap;
+  const int grid = elementwise_ctas(n, sms);
   for (int level = 1; level <= 3; ++level) {
-    if (launch_l1_level(la, level, (int)grid, st) != cudaSuccess) return S3TTV_ECUDA;
+    if (launch_l1_level(la, level, grid, st) != cudaSuccess) return S3TTV_ECUDA;
   }
   if (launch_soft_threshold(x, out, n, sc, 0, st) != cudaSuccess) return S3TTV_ECUDA;
   L1State state;

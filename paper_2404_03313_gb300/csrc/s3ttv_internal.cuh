@@ -114,6 +114,19 @@ struct L1Args {
   unsigned *hcnt;         // [2][kHistBins]
   double *hsum;           // [2][kHistBins]
 };
+// CTAs (512 threads, float4 pieces) of the elementwise and threshold kernels over n
+// elements: at most two per SM, because each adds its histogram into the global one,
+// but in multiples of that enough that none takes more than 2 M elements: a CTA's
+// integer bin sums (l1_select.cuh) stay below 2^32 up to 4 M.  (At most kMaxGrid.)
+constexpr int kMaxGrid = 4096;
+inline int elementwise_ctas(long long n, int num_sms) {
+  const long long cap = 2ll * (num_sms > 0 ? num_sms : 1), waves = n / (cap << 21) + 1;
+  const long long most = kMaxGrid / cap > 0 ? kMaxGrid / cap * cap : kMaxGrid;
+  long long g = (n + 2047) / 2048;
+  if (g > cap * waves) g = cap * waves;
+  if (g > most) g = most;
+  return g < 1 ? 1 : (int)g;
+}
 cudaError_t launch_l1_level(const L1Args &a, int level, int grid, cudaStream_t st);
 cudaError_t launch_soft_threshold(const float *x, float *out, long long n, const Scalars *sc,
                                   int prob, cudaStream_t st);

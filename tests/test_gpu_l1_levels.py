@@ -46,3 +46,17 @@ def test_l1_ball_equal_values_and_zeros(solver):
         out, _ = solver.l1_ball(torch.from_numpy(x).cuda(), radius)
         ref = O.proj_l1_ball(x.astype(np.float64), radius)
         assert np.linalg.norm(out.cpu().numpy() - ref) <= 1e-5 * np.linalg.norm(ref)
+
+
+def test_l1_ball_largest(solver):
+    """Every element in one bin of every level, its low bits all ones: the bin sums of
+    1.4e9 elements pass 2^32 per CTA unless the grid grows with n.  The projection of a
+    constant c to radius n r is the constant r."""
+    n = 1_400_000_000
+    if torch.cuda.mem_get_info()[0] < 12e9:
+        pytest.skip("needs 12 GB")
+    x = torch.full((n,), float(np.nextafter(np.float32(2.0), np.float32(0.0))), device="cuda")
+    out, tau = solver.l1_ball(x, float(n), out=x)
+    assert abs(tau - (2.0 - 2.0 ** -23 - 1.0)) <= 1e-5
+    lo, hi = torch.aminmax(out)
+    assert abs(float(lo) - 1.0) <= 1e-5 and abs(float(hi) - 1.0) <= 1e-5
