@@ -796,11 +796,11 @@ int ensure_events(s3ttv_ctx *ctx, int passes) {
 int collect_events(s3ttv_ctx *ctx, int passes) {
   for (int p = 0; p < passes; ++p) {
     cudaEvent_t *e = ctx->ev + (size_t)kEvPerPass * p;
-    for (int c = 0; c < S3TTV_KERNEL_CLASSES; ++c) {
+    for (int c = 0; c < S3TTV_KERNEL_FINALIZE; ++c) {  // (which launches nothing)
       float ms = 0.f;
       CU(cudaEventElapsedTime(&ms, e[c], e[c + 1]));
       ctx->prof_ms[c] += ms;
-      ctx->prof_n[c] += c == S3TTV_KERNEL_L1_SEARCH ? 2 : c == S3TTV_KERNEL_FINALIZE ? 0 : 1;
+      ctx->prof_n[c] += c == S3TTV_KERNEL_L1_SEARCH ? 2 : 1;
     }
   }
   return S3TTV_OK;
