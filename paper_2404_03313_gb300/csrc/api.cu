@@ -702,10 +702,10 @@ int enqueue_pass(s3ttv_ctx *ctx, int par, int grid_e, const BdShape &bd,
   ph.next("block dual (steps 8-11)");
   if (ctx->reg == S3TTV_REG_SSTV) {
     CU(launch_sstv_dual(ctx->ubar, ctx->Y, ctx->Y + dm.Np, ctx->Zv[par ^ 1], ctx->Zh[par ^ 1], dm,
-                        (float)ctx->gam[3], grid_e, st));
+                        (float)ctx->gam[3], ctx->sc, grid_e, st));
   } else if (is_hsstv(ctx)) {
     CU(launch_hsstv_dual(ctx->ubar, ctx->Y, ctx->Zv[par ^ 1], ctx->Zh[par ^ 1], dm, (float)ctx->gam[3],
-                         ctx->hsstv_omega, ctx->reg == S3TTV_REG_HSSTV2, grid_e, st));
+                         ctx->hsstv_omega, ctx->reg == S3TTV_REG_HSSTV2, ctx->sc, grid_e, st));
   } else {
   if (part == 1) {
     ctx->launches += 3;  // primal, xfield with the second level, third level

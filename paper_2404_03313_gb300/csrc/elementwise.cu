@@ -409,10 +409,13 @@ cudaError_t launch_dual(const DualArgs &a, int grid, cudaStream_t st) {
 // norms): Y' = Y + gamma_Y (D_v D_s ubar, D_h D_s ubar), and the conjugate prox
 // of the l1 norm (eq. ProxConjugate) is the projection onto the unit l_inf
 // ball, Y = clip(Y', -1, 1).  Y = (Yv, Yh) are internal cubes, and
-// Z = sum_l P_l^T Y_l becomes Y itself: written to (Zv, Zh).
+// Z = sum_l P_l^T Y_l becomes Y itself: written to (Zv, Zh).  Nothing moves once the
+// stop rule has fired: the passes enqueued beyond it would step Y in place.
 __global__ void sstv_dual_kernel(const float *__restrict__ ubar, float *__restrict__ Yv, float *__restrict__ Yh,
-                                 float *__restrict__ Zv, float *__restrict__ Zh, Dims dm, float gY) {
+                                 float *__restrict__ Zv, float *__restrict__ Zh, Dims dm, float gY,
+                                 const Scalars *sc) {
   chained();
+  if (sc->done) return;
   const int N3p = dm.N3p, C4 = N3p >> 2, N2 = dm.N2;
   const int nch = (int)(dm.P * C4);
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nch; c += gridDim.x * blockDim.x) {
@@ -453,8 +456,10 @@ __global__ void sstv_dual_kernel(const float *__restrict__ ubar, float *__restri
 // voxel's four entries (l12 = 1: scale the 4-vector into the unit l2 ball).
 // Y holds four internal cubes; the second-order pair is also written to Z.
 __global__ void hsstv_dual_kernel(const float *__restrict__ ubar, float *__restrict__ Y, float *__restrict__ Zv,
-                                  float *__restrict__ Zh, Dims dm, float gY, float omega, int l12) {
+                                  float *__restrict__ Zh, Dims dm, float gY, float omega, int l12,
+                                  const Scalars *stop) {
   chained();
+  if (stop->done) return;
   const int N3p = dm.N3p, C4 = N3p >> 2, N2 = dm.N2;
   const int nch = (int)(dm.P * C4);
   const size_t Np = (size_t)dm.Np;
@@ -501,13 +506,13 @@ __global__ void hsstv_dual_kernel(const float *__restrict__ ubar, float *__restr
 }
 
 cudaError_t launch_hsstv_dual(const float *ubar, float *Y, float *Zv, float *Zh, Dims dm, float gY, float omega,
-                              int l12, int grid, cudaStream_t st) {
-  return launch_chained(hsstv_dual_kernel, 4 * grid, 256, 0, st, ubar, Y, Zv, Zh, dm, gY, omega, l12);
+                              int l12, const Scalars *sc, int grid, cudaStream_t st) {
+  return launch_chained(hsstv_dual_kernel, 4 * grid, 256, 0, st, ubar, Y, Zv, Zh, dm, gY, omega, l12, sc);
 }
 
 cudaError_t launch_sstv_dual(const float *ubar, float *Yv, float *Yh, float *Zv, float *Zh, Dims dm, float gY,
-                             int grid, cudaStream_t st) {
-  return launch_chained(sstv_dual_kernel, 4 * grid, 256, 0, st, ubar, Yv, Yh, Zv, Zh, dm, gY);
+                             const Scalars *sc, int grid, cudaStream_t st) {
+  return launch_chained(sstv_dual_kernel, 4 * grid, 256, 0, st, ubar, Yv, Yh, Zv, Zh, dm, gY, sc);
 }
 
 cudaError_t launch_pad_cube(const float *src, float *dst, Dims dm, float scale, cudaStream_t st) {

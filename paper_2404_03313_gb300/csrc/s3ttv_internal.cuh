@@ -230,13 +230,13 @@ cudaError_t launch_Y_to_external(const float *in, float *ext, Dims dm, int k, cu
 cudaError_t launch_xfield(const float *ubar, float *Fv, float *Fh, Dims dm, int grid, cudaStream_t st,
                          int open_s, int first_order, float *Fs = nullptr, const L1Args *l1 = nullptr);
 // SSTV's dual step: Y = clip(Y + gamma_Y D D_s ubar, -1, 1) on the cube pair
-// (Yv, Yh), and Z = Y
+// (Yv, Yh), and Z = Y, unless the stop rule has fired (sc)
 cudaError_t launch_sstv_dual(const float *ubar, float *Yv, float *Yh, float *Zv, float *Zh, Dims dm, float gY,
-                             int grid, cudaStream_t st);
+                             const Scalars *sc, int grid, cudaStream_t st);
 // HSSTV's dual step on four cubes Y (second-order pair then omega-weighted
 // first-order pair): l1 (l12 = 0) or per-voxel l1,2 (l12 = 1) conjugate prox
 cudaError_t launch_hsstv_dual(const float *ubar, float *Y, float *Zv, float *Zh, Dims dm, float gY, float omega,
-                              int l12, int grid, cudaStream_t st);
+                              int l12, const Scalars *sc, int grid, cudaStream_t st);
 cudaError_t launch_Z_from_Y(const float *Y, float *Zv, float *Zh, Dims dm, int k, cudaStream_t st,
                             float *Zs = nullptr);
 cudaError_t launch_init_scalars(Scalars *sc, double alpha, double beta, cudaStream_t st);

@@ -1,0 +1,58 @@
+"""GPU: the state after the stop rule has fired does not depend on how many passes
+were enqueued before the host read the flag (S3TTV_OPT_CHECK_EVERY), for every
+regulariser, nor does a run continued from it.
+
+Tolerance: the two runs execute the same passes; what may differ is the order of
+the FP64 histogram sums (1e-16 relative, which may move a threshold by one FP32
+rounding) and of the FP32 additions into Z of the block regularisers (k^2 = 4
+terms, 4 u relative), over a few dozen passes: 1e-5 relative L2.  A dual step that
+runs on past the stop moves Y by more than 1e-2.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-5
+
+
+@pytest.fixture(scope="module")
+def P():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2404_03313_gb300 as P
+    P.library()
+    return P
+
+
+@pytest.mark.parametrize("reg", ["REG_S3TTV", "REG_STV", "REG_SSTV", "REG_HSSTV1", "REG_HSSTV2", "REG_SSST"])
+def test_state_after_the_stop_does_not_depend_on_check_every(P, reg):
+    v = np.random.default_rng(3).uniform(0, 1, (14, 11, 9)).astype(np.float32)
+    args = (0.05 * v.size ** 0.5, 0.02 * v.size, 0.02 * v.size, 2)
+
+    def solver(check_every):
+        s = P.Solver(0)
+        s.set_option(P.OPT_REGULARIZER, getattr(P, reg))
+        s.set_option(P.OPT_CHECK_EVERY, check_every)
+        s.setup(v, *args)
+        s.iterate(3)
+        return s
+
+    # a tolerance that pass j + 1 of the run is the first to meet, between two looks at the flag
+    with solver(1) as s:
+        rels = [s.iterate(1)["rel_change"] for _ in range(60)]
+    j = next(i for i in range(1, 60) if (i + 1) % 16 and rels[i] < 0.999 * min(rels[:i]))
+    tol = 0.5 * (rels[j] + min(rels[:j]))
+    out = {}
+    for ce in (1, 16):
+        with solver(ce) as s:
+            info = s.iterate(100, tol)
+            stopped = {n: s.get_state(n) for n in ("u", "s", "t", "y2", "y3", "Y")}
+            s.iterate(5)
+            out[ce] = info, stopped, {n: s.get_state(n) for n in ("u", "Y")}
+    assert out[1][0]["iters"] == out[16][0]["iters"] == j + 1
+    for one, many in zip(out[1][1:], out[16][1:]):
+        for n in one:
+            err = np.linalg.norm(one[n].astype(np.float64) - many[n]) / max(np.linalg.norm(one[n]), 1e-30)
+            assert err <= TOL, (n, err)
