@@ -94,7 +94,12 @@ __global__ void __launch_bounds__(256) sam_kernel(const float *u, const float *r
 // difference stand for the five of x and y: mx my = (p^2 - m^2) / 4,
 // mx^2 + my^2 = (p^2 + m^2) / 2, and likewise for the (co)variances.
 // Bound by the FP64 rate: about 92 operations and one division per voxel in place
-// of 121 taps of seven; 15.98 -> 2.35 ms at 256 x 256 x 128.
+// of 121 taps of seven; 15.98 -> 2.35 ms at 256 x 256 x 128.  Where fewer than
+// kSsimCols output columns are left, the warps without one only help to fill the rows
+// (400000 x 11 x 32: 65 -> 13.7 ms, 200000 x 12 x 4: 32.8 -> 7.7 ms with it and with
+// as many row chunks as fill the SMs).
+// A CTA is one group of bands, then one tile of columns, then one chunk of rows, all
+// on grid.x: the other grid dimensions end at 65535, which a wide image exceeds.
 constexpr int kSsimCols = 8;
 constexpr int kSsimRowCols = kSsimCols + kSsimTaps - 1;
 struct SsimWeights {
@@ -102,13 +107,17 @@ struct SsimWeights {
 };
 
 __global__ void __launch_bounds__(32 * kSsimCols, 2) ssim_kernel(const float *u, const float *ref, int N1, int N2, int N3,
-                                                               int b0, int nb, int rows, SsimWeights sw, double *out) {
+                                                               int b0, int nb, int rows, int gx, int gy, SsimWeights sw,
+                                                               double *out) {
   __shared__ double row[2][kSsimRowCols][4][32];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
   const int Hv = N1 - kSsimTaps + 1, Wv = N2 - kSsimTaps + 1;
-  const int b = min(b0 + (int)blockIdx.x * 32 + lane, b0 + nb - 1);  // lanes past the last band repeat it
-  const int j0 = blockIdx.y * kSsimCols, i0 = blockIdx.z * rows;
-  const int nin = min(rows, Hv - i0) + kSsimTaps - 1;  // input rows of this CTA
+  const int xg = blockIdx.x % gx, xr = blockIdx.x / gx;
+  const int b = min(b0 + xg * 32 + lane, b0 + nb - 1);  // lanes past the last band repeat it
+  const int j0 = xr % gy * kSsimCols, i0 = xr / gy * rows;
+  const int ncol = min(kSsimRowCols, N2 - j0);  // input columns of this CTA
+  const bool mine = j0 + wp < Wv;               // this warp has an output column
+  const int nout = min(rows, Hv - i0), nin = nout + kSsimTaps - 1;  // output and input rows of this CTA
   constexpr int LD = (kSsimRowCols + kSsimCols - 1) / kSsimCols;
   float xs[LD], ys[LD];
   auto fetch = [&](int r) {  // this warp's columns of input row r
@@ -116,8 +125,8 @@ __global__ void __launch_bounds__(32 * kSsimCols, 2) ssim_kernel(const float *u,
     for (int e = 0; e < LD; ++e) {
       const int c = wp + e * kSsimCols;
       xs[e] = ys[e] = 0.f;
-      if (c < kSsimRowCols && r < nin) {
-        const size_t o = ((size_t)(i0 + r) * N2 + min(j0 + c, N2 - 1)) * N3 + b;
+      if (c < ncol && r < nin) {
+        const size_t o = ((size_t)(i0 + r) * N2 + j0 + c) * N3 + b;
         xs[e] = ref[o];
         ys[e] = u[o];
       }
@@ -135,7 +144,7 @@ __global__ void __launch_bounds__(32 * kSsimCols, 2) ssim_kernel(const float *u,
 #pragma unroll
         for (int e = 0; e < LD; ++e) {
           const int c = wp + e * kSsimCols;
-          if (c < kSsimRowCols) {
+          if (c < ncol) {
             const double x = xs[e], y = ys[e], p = x + y, m = x - y;
             buf[c][0][lane] = p;
             buf[c][1][lane] = m;
@@ -145,6 +154,7 @@ __global__ void __launch_bounds__(32 * kSsimCols, 2) ssim_kernel(const float *u,
         }
         fetch(r + 1);
         __syncthreads();
+        if (!mine) continue;  // (to the next row's barrier)
         double h[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
         for (int c = 0; c < kSsimTaps; ++c)
@@ -153,6 +163,7 @@ __global__ void __launch_bounds__(32 * kSsimCols, 2) ssim_kernel(const float *u,
         // output row o sits in slot o mod 11 and takes input row r with weight r - o
 #pragma unroll
         for (int k = 0; k < kSsimTaps; ++k) {
+          if ((unsigned)(r - k) >= (unsigned)nout) continue;  // not an output row of this CTA
           const int s = (ph - k + kSsimTaps) % kSsimTaps;
 #pragma unroll
           for (int q = 0; q < 4; ++q) acc[s][q] = k == 0 ? sw.w[0] * h[q] : fma(sw.w[k], h[q], acc[s][q]);
@@ -170,9 +181,9 @@ __global__ void __launch_bounds__(32 * kSsimCols, 2) ssim_kernel(const float *u,
   }
   __syncthreads();
   double *red = &row[0][0][0][0];
-  red[wp * 32 + lane] = j0 + wp < Wv ? total : 0.0;
+  red[wp * 32 + lane] = total;  // (zero without a column)
   __syncthreads();
-  if (wp == 0 && (int)blockIdx.x * 32 + lane < nb) {
+  if (wp == 0 && xg * 32 + lane < nb) {
     double s = 0.0;
     for (int w = 0; w < kSsimCols; ++w) s += red[w * 32 + lane];
     atomicAdd(out + (b - b0), s);
@@ -423,16 +434,19 @@ cudaError_t launch_ssim(const float *u, const float *ref, int N1, int N2, int N3
   // first 10 rows only feed its windows, at a bit over half a row's work
   int rows = Hv;
   double best = 1e300;
-  for (int n = 1; n <= Hv && n <= 64; ++n) {
-    const int r = (Hv + n - 1) / n;
-    const long long ctas = (long long)gx * gy * ((Hv + r - 1) / r), slots = 2LL * num_sms;
+  const long long tiles = (long long)gx * gy, slots = 2LL * num_sms;
+  for (long long n = 1; n <= Hv && (n == 1 || tiles * n <= 16 * slots); n += n < 64 ? 1 : n / 16) {
+    const int r = (int)((Hv + n - 1) / n);
+    const long long ctas = tiles * ((Hv + r - 1) / r);
     const double cost = (double)((ctas + slots - 1) / slots) * (r + 6.0);
     if (cost < best) {
       best = cost;
       rows = r;
     }
   }
-  ssim_kernel<<<dim3(gx, gy, (Hv + rows - 1) / rows), 32 * kSsimCols, 0, st>>>(u, ref, N1, N2, N3, b0, nb, rows, sw, out);
+  const long long ctas = tiles * ((Hv + rows - 1) / rows);
+  if (ctas > 0x7fffffffLL) return cudaErrorInvalidValue;
+  ssim_kernel<<<(unsigned)ctas, 32 * kSsimCols, 0, st>>>(u, ref, N1, N2, N3, b0, nb, rows, gx, gy, sw, out);
   return cudaGetLastError();
 }
 
