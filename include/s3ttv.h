@@ -506,6 +506,16 @@ int s3ttv_net_create(s3ttv_net **out, int device, void *cuda_stream);
 void s3ttv_net_destroy(s3ttv_net *net); /* NULL-safe */
 const char *s3ttv_net_last_error(const s3ttv_net *net);
 
+/* Options of a network. */
+enum {
+  S3TTV_NET_OPT_WAIT_NS = 1 /* time limit, in nanoseconds, of each wait inside the
+                               convolution kernels (default 4e9, at most 1e11); a wait
+                               that runs out ends the call with S3TTV_ECUDA and leaves
+                               the network usable; 0: no wait is sat out, and the call
+                               ends so in any case (for failure tests)                 */
+};
+int s3ttv_net_set_option(s3ttv_net *net, int key, double value);
+
 /* Load parameters (param_count floats) and reset the Adam state. */
 int s3ttv_net_set_params(s3ttv_net *net, const float *theta);
 /* Copy the current FP32 parameters out (param_count floats). */

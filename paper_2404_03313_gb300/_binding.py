@@ -32,6 +32,7 @@ OPT_NVTX = 15
 OPT_JACOBI_POLISH_TOL = 16
 OPT_FIRST_ORDER = 17
 OPT_BATCH_WORKLIST = 18
+NET_OPT_WAIT_NS = 1
 REG_S3TTV, REG_STV, REG_SSTV, REG_HSSTV1, REG_HSSTV2, REG_SSST = 0, 1, 2, 3, 4, 5
 KERNEL_CLASSES = ("primal", "l1_search", "block_dual", "dual", "finalize")
 STATE = {"u": 0, "s": 1, "t": 2, "y2": 3, "y3": 4, "Y": 5}
@@ -88,6 +89,7 @@ SIGNATURES = {
     "s3ttv_net_create": (_c_int, [_P(_vp), _c_int, _vp]),
     "s3ttv_net_destroy": (None, [_vp]),
     "s3ttv_net_last_error": (ctypes.c_char_p, [_vp]),
+    "s3ttv_net_set_option": (_c_int, [_vp, _c_int, _c_d]),
     "s3ttv_net_set_params": (_c_int, [_vp, _vp]),
     "s3ttv_net_get_params": (_c_int, [_vp, _vp]),
     "s3ttv_net_forward": (_c_int, [_vp, _vp, _c_int, _c_int, _c_int, _c_int, _vp, _vp, _vp]),
@@ -485,6 +487,9 @@ class WarmStartNet:
             msg = self._lib.s3ttv_net_last_error(self._h).decode(errors="replace")
             raise S3TTVError(rc, f"{what}: {msg}")
         return rc
+
+    def set_option(self, key, value):
+        self._check(self._lib.s3ttv_net_set_option(self._h, int(key), float(value)), "set_option")
 
     def set_params(self, theta):
         _sync_torch(theta)

@@ -517,7 +517,10 @@ struct s3ttv_net {
   float *theta = nullptr, *grad = nullptr, *m1 = nullptr, *m2 = nullptr, *hp = nullptr;
   bf16 *wf = nullptr, *wb = nullptr;
   double *loss = nullptr;
-  int *err_flag = nullptr;  // host memory the kernels write when a wait of theirs runs out
+  // written by the kernels when a wait of theirs runs out: host memory, read by
+  // finish(), and device memory
+  int *err_flag = nullptr, *bad = nullptr;
+  unsigned long long wait_ns = kWaitNs;
   long long adam_t = 0;
   bool have_params = false;
   // shape-dependent workspace
@@ -579,13 +582,13 @@ int grid_for(const s3ttv_net *net, long long items, int threads) {
 
 cudaError_t launch_conv(const s3ttv_net *net, const bf16 *x0, int c0, const bf16 *x1, int c1, const bf16 *w,
                         const float *bias, const bf16 *mask, bf16 *y, int cout, bool relu, Vol g) {
-  ConvArgs a{x0, x1, w, bias, mask, y, c0, c1, cout, relu ? 1 : 0, g, net->err_flag};
+  ConvArgs a{x0, x1, w, bias, mask, y, c0, c1, cout, relu ? 1 : 0, g, net->err_flag, net->bad, net->wait_ns};
   return conv_launch(a, net->num_sms, net->stream);
 }
 
 cudaError_t launch_wgrad(const s3ttv_net *net, const bf16 *G, int cout, const bf16 *x0, int c0, const bf16 *x1,
                          int c1, float *dw, float *db, Vol g) {
-  WgradTcArgs a{G, x0, x1, dw, db, c0, c1, cout, g, net->err_flag};
+  WgradTcArgs a{G, x0, x1, dw, db, c0, c1, cout, g, net->err_flag, net->bad, net->wait_ns};
   return wgrad_launch(a, net->num_sms, net->stream);
 }
 
@@ -689,7 +692,8 @@ int run_forward(s3ttv_net *net, const float *v, const Vol &g0, float *const *out
   NCU(launch_conv(net, net->e2b, 64, net->bb, 128, wf(net, 6), bias(net, 6), nullptr, net->d2a, 64, true, g1));
   NCU(launch_conv(net, net->d2a, 64, nullptr, 0, wf(net, 7), bias(net, 7), nullptr, net->d2b, 64, true, g1));
   NCU(launch_conv(net, net->e1b, 32, net->d2b, 64, wf(net, 8), bias(net, 8), nullptr, net->d1a, 32, true, g0));
-  ConvArgs last{net->d1a, nullptr, wf(net, 9), bias(net, 9), nullptr, net->d1b, 32, 0, 32, 1, g0, net->err_flag};
+  ConvArgs last{net->d1a, nullptr, wf(net, 9), bias(net, 9), nullptr, net->d1b, 32, 0, 32, 1, g0,
+                net->err_flag, net->bad, net->wait_ns};
   if (out) {
     last.y = nullptr;
     last.hp = net->hp;
@@ -773,6 +777,7 @@ int finish(s3ttv_net *net) {
   NCU(cudaStreamSynchronize(net->stream));
   if (*(volatile int *)net->err_flag) {
     *net->err_flag = 0;
+    NCU(cudaMemsetAsync(net->bad, 0, sizeof(int), net->stream));
     return nfail(net, S3TTV_ECUDA, "a convolution kernel's wait ran out of time");
   }
   return S3TTV_OK;
@@ -832,6 +837,8 @@ int s3ttv_net_create(s3ttv_net **out, int device, void *stream) {
   ok = ok && cudaMalloc(&net->wb, P * sizeof(bf16)) == cudaSuccess;
   ok = ok && cudaMalloc(&net->hp, (kHeadIn * kHeadOut + kHeadOut) * sizeof(float)) == cudaSuccess;
   ok = ok && cudaMalloc(&net->loss, sizeof(double)) == cudaSuccess;
+  ok = ok && cudaMalloc(&net->bad, sizeof(int)) == cudaSuccess;
+  ok = ok && cudaMemsetAsync(net->bad, 0, sizeof(int), net->stream) == cudaSuccess;
   ok = ok && cudaHostAlloc(&net->err_flag, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
@@ -854,7 +861,7 @@ void s3ttv_net_destroy(s3ttv_net *net) {
     Guard gd(net->device);
     if (net->stream) cudaStreamSynchronize(net->stream);
     void *bufs[] = {net->theta, net->grad, net->m1, net->m2, net->wf, net->wb, net->hp, net->loss, net->arena,
-                    net->stage};
+                    net->stage, net->bad};
     for (void *b : bufs)
       if (b) cudaFree(b);
     if (net->err_flag) cudaFreeHost(net->err_flag);
@@ -864,6 +871,14 @@ void s3ttv_net_destroy(s3ttv_net *net) {
 }
 
 const char *s3ttv_net_last_error(const s3ttv_net *net) { return net ? net->err : "null network"; }
+
+int s3ttv_net_set_option(s3ttv_net *net, int key, double value) {
+  if (!net) return S3TTV_EINVAL;
+  if (key != S3TTV_NET_OPT_WAIT_NS) return nfail(net, S3TTV_EINVAL, "unknown option %d", key);
+  if (!(value >= 0 && value <= 1e11)) return nfail(net, S3TTV_EINVAL, "the time limit must be in [0, 1e11] ns");
+  net->wait_ns = (unsigned long long)value;
+  return S3TTV_OK;
+}
 
 int s3ttv_net_set_params(s3ttv_net *net, const float *theta) {
   if (!net || !theta) return S3TTV_EINVAL;

@@ -27,7 +27,8 @@
 // slice) stages; with 32 input channels all of them once, a CTA keeps its tile of
 // output channels); warps 11-18 copy planes (cp.async with zero fill outside the volume, nearest upsampling
 // by halving the coordinates).  Every wait has a time limit, after which the CTA
-// sets the error flag and ends.
+// ends its roles, waits for its MMAs and copies in flight, frees its TMEM, sets the
+// error flags and ends.
 #include "unet_conv.cuh"
 
 #include "chain.cuh"
@@ -47,7 +48,6 @@ constexpr int kMaxAStages = 4, kMaxWStages = 16, kMaxSlots = 8;
 constexpr int kTmemCols = 512;
 constexpr int kSmemMax = 227 * 1024 - 2048;
 constexpr int kSmemMin = 120 * 1024;  // one CTA per SM: each takes all of TMEM
-constexpr unsigned long long kWaitNs = 4000000000ull;
 
 // Input channels per weight stage, and whether a CTA keeps all its weights in
 // shared memory (9 stages of 6 or 12 KB at 32 input channels).
@@ -90,16 +90,16 @@ __device__ __forceinline__ unsigned long long now_ns() {
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
   return t;
 }
-// Wait for a barrier's phase; false when the time limit or another role's
+// Wait for a barrier's phase; false when the time limit (in ns) or another role's
 // failure (stop) ends the wait.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *stop) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *stop, unsigned long long limit) {
   if (mbar_try(bar, parity)) return true;
   const unsigned long long t0 = now_ns();
   while (true) {
     for (int i = 0; i < 32; ++i)
       if (mbar_try(bar, parity)) return true;
     if (*stop) return false;
-    if (now_ns() - t0 > kWaitNs) {
+    if (now_ns() - t0 > limit) {
       *stop = 1;
       return false;
     }
@@ -126,6 +126,18 @@ __device__ __forceinline__ bool elect_one() {
   uint32_t r;
   asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.b32 %0, 1, 0, p;\n}\n" : "=r"(r));
   return r != 0;
+}
+// Wait for what is in flight, so that no MMA or copy outlives the CTA, its shared
+// memory or its TMEM, whichever role failed.
+__device__ __forceinline__ void mbar_drain(uint32_t bar, uint32_t parity, volatile int *stop) {
+  for (int i = 0; i < 32; ++i)
+    if (mbar_try(bar, parity)) return;
+  const unsigned long long t0 = now_ns();  // (reading the clock takes about a microsecond)
+  while (!mbar_try(bar, parity))
+    if (now_ns() - t0 > kWaitNs) {
+      *stop = 1;
+      return;
+    }
 }
 // The operand descriptors come as their low and high words: the high words are
 // constants and only the low ones (start address) move.  add = 0: D = A B, else
@@ -201,7 +213,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
   __shared__ __align__(16) float s_bias[192];
   __shared__ __align__(16) float s_head[100];  // the head's weights and biases
   __shared__ uint32_t s_tmem;
-  __shared__ int s_stop;
+  __shared__ int s_stop[2];  // a wait has run out; the weight copies have ended
   const int tid = threadIdx.x, lane = tid & 31;
   // broadcasts, so that the compiler knows the role and TMEM address as warp-uniform
   // and keeps the MMA loop's operands in uniform registers
@@ -218,7 +230,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
   auto w_empty = [&](int s) { return bar0 + 8u * (2 * kMaxAStages + kMaxWStages + s); };
   auto c_full = [&](int s) { return bar0 + 8u * (2 * kMaxAStages + 2 * kMaxWStages + s); };
   auto c_empty = [&](int s) { return bar0 + 8u * (2 * kMaxAStages + 2 * kMaxWStages + kMaxSlots + s); };
-  const uint32_t drained = c_empty(kMaxSlots);  // (two) after a failure: the MMAs issued so far are done
+  const uint32_t drained = c_empty(kMaxSlots);  // (two): a tile's MMAs are done
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&s_tmem)),
@@ -242,7 +254,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
     mbar_init(drained, 1);
     mbar_init(drained + 8, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    s_stop = 0;
+    s_stop[0] = a.wait_ns == 0;  // no wait is sat out
+    s_stop[1] = 0;
   }
   for (int i = tid; i < a.cout; i += kThreads) s_bias[i] = a.bias ? a.bias[i] : 0.f;
   if (a.hp && tid < 99) s_head[tid] = a.hp[tid];
@@ -250,7 +263,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
   __syncthreads();
   fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
-  volatile int *stop = &s_stop;
+  volatile int *stop = s_stop;
+  const unsigned long long limit = a.wait_ns;
 
   if (warp < kEpiWarps) {
     // ---- epilogue: slot k of the ring holds output plane k, k + S, ... of this CTA ----
@@ -263,7 +277,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
     for (int u = u0; u < pl.units && ok; u += du) {
       const Unit t = unit_at(u, pl, g);
       for (int z = t.z0; z < t.z1; ++z) {
-        ok = __all_sync(0xffffffffu, mbar_wait(c_full(slot), phase, stop));
+        ok = __all_sync(0xffffffffu, mbar_wait(c_full(slot), phase, stop, limit));
         if (!ok) break;
         fence_after();
         // this warp's blocks of the tile are first, first + 2, ...; the slot is free
@@ -360,8 +374,10 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
       int as = 0, ws = 0, slot0 = 0;        // slot0: the slot of the unit's first output plane
       uint32_t aph = 0, wph = 0, cph = 1;   // cph: the parity to wait for in the ring turn slot0 is in
       bool ok = true;
+      // (a wait for weights that fails ends this loop at its next other wait, or lets it run
+      // on to its end over whatever lies there: the result is reported as failed)
       if (RES)
-        for (int st = 0; st < 9; ++st) mbar_wait(w_full(st), 0, stop);
+        for (int st = 0; st < 9; ++st) mbar_wait(w_full(st), 0, stop, limit);
       for (int u = u0; u < pl.units && ok; u += du) {
         const Unit t = unit_at(u, pl, g);
         for (int p = t.p0; p <= t.p1; ++p) {
@@ -371,9 +387,9 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
             if (p != max(z - 1, 0)) continue;  // not the first plane that adds into z
             // c_empty(s) completes its phase k - 1 when the slot is free for its k-th use
             const int k = slot0 + (z - t.z0);
-            got = mbar_wait(c_empty(k & (S - 1)), cph ^ (uint32_t)((k >> pl.sh) & 1), stop) && got;
+            got = mbar_wait(c_empty(k & (S - 1)), cph ^ (uint32_t)((k >> pl.sh) & 1), stop, limit) && got;
           }
-          got = mbar_wait(a_full(as), aph, stop) && got;
+          got = mbar_wait(a_full(as), aph, stop, limit) && got;
           ok = __all_sync(0xffffffffu, got);
           if (!ok) break;
           fence_after();
@@ -392,7 +408,12 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
           for (int yx = 0; yx < 9; ++yx) {
 #pragma unroll
             for (int sl = 0; sl < NS; ++sl) {
-              if (!RES) mbar_wait(w_full(ws), wph, stop);  // (a wait that fails shows at the next plane)
+              // (a failed wait for weights still sits the copy out, unless none will come: its
+              // stage may not be armed again before it lands; nothing else is checked here, where
+              // a vote or a flag carried along cost 2 to 10%)
+              if (!RES && !mbar_wait(w_full(ws), wph, stop, limit))
+                for (unsigned i = 0; i < (1u << 26) && !mbar_try(w_full(ws), wph) && !stop[1]; ++i) {
+                }
               const uint32_t blo = RES ? blo0 + wstep * yx : uniform(blo0 + wstep * ws);
               const uint32_t a0 = tap + (uint32_t)(sl * (CS / 16)) * ak;
               if (issue) {
@@ -437,12 +458,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
         cph ^= (uint32_t)((k >> pl.sh) & 1);
         slot0 = k & (S - 1);
       }
-      if (!ok && issue) {  // drain what was issued before TMEM is given back
-        mma_commit(drained + 8u * sub);
-        const unsigned long long t0 = now_ns();
-        while (!mbar_try(drained + 8u * sub, 0) && now_ns() - t0 < kWaitNs) {
-        }
-      }
+      if (issue) mma_commit(drained + 8u * sub);
     }
   } else if (warp == kWWarp) {
     if (lane == 0) {
@@ -465,7 +481,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
           const Unit t = unit_at(u, pl, g);
           for (int p = t.p0; p <= t.p1 && ok; ++p)
             for (int st = 0; st < 9 * NS; ++st) {
-              if (!(ok = mbar_wait(w_empty(ws), ph, stop))) break;
+              ok = mbar_wait(w_empty(ws), ph, stop, limit);
+              if (!ok) break;
               mbar_expect(w_full(ws), w_bytes);
               bulk_copy(sW + w_bytes * ws, stage_src(st / NS, st % NS), w_bytes, w_full(ws));
               ++issued;
@@ -476,13 +493,9 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
             }
         }
       }
-      if (RES || !ok) {  // copies in flight land before the CTA ends
-        const unsigned first = issued > (unsigned)pl.w_stages ? issued - pl.w_stages : 0u;
-        const unsigned long long t0 = now_ns();
-        for (unsigned i = first; i < issued; ++i)
-          while (!mbar_try(w_full(i % pl.w_stages), (i / pl.w_stages) & 1) && now_ns() - t0 < kWaitNs) {
-          }
-      }
+      for (unsigned i = issued > (unsigned)pl.w_stages ? issued - pl.w_stages : 0u; i < issued; ++i)
+        mbar_drain(w_full(i % pl.w_stages), (i / pl.w_stages) & 1, stop);
+      stop[1] = 1;
     }
   } else {
     // ---- plane copies ----
@@ -512,7 +525,7 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
         off[i] = in ? ((y >> hs) * Ws + (x >> hs)) * C : -1;
       }
       for (int p = t.p0; p <= t.p1; ++p) {
-        ok = __all_sync(0xffffffffu, mbar_wait(a_empty(as), ph, stop));
+        ok = __all_sync(0xffffffffu, mbar_wait(a_empty(as), ph, stop, limit));
         if (!ok) break;
         const uint32_t dst = sA + a_bytes * as + (uint32_t)q * pl.lbo + (uint32_t)v0 * 16;
         const bf16 *plane = base + ((size_t)t.b * Ds + (p >> hs)) * Hs * Ws * C;
@@ -546,10 +559,15 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
   fence_before();
   __syncthreads();
   if (warp == 0) {
+    if (*stop)  // (otherwise the accumulators read out say as much)
+      for (int j = 0; j < J; ++j) mbar_drain(drained + 8u * j, 0, stop);
     fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTmemCols));
   }
-  if (tid == 0 && *stop) *reinterpret_cast<volatile int *>(a.err) = 1;
+  if (tid == 0 && *stop) {
+    *reinterpret_cast<volatile int *>(a.err) = 1;
+    *a.bad = 1;
+  }
 }
 
 // ---------------------------------------------------------------- weight gradient
@@ -609,7 +627,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wgrad_tc_kernel(WgradTcArgs a, W
     }
     mbar_init(done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    s_stop = 0;
+    s_stop = a.wait_ns == 0;  // no wait is sat out
   }
   // the fourth plane of every stage: channel 0 one, the others zero
   for (int i = tid; i < kWStages * 4 * (kWX / 16); i += kWThreads) {
@@ -652,7 +670,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wgrad_tc_kernel(WgradTcArgs a, W
     for (int u = first; u < pl.bricks; u += pl.per) {
       int b, x0, y0, z0;
       brick(u, b, x0, y0, z0);
-      ok = __all_sync(0xffffffffu, mbar_wait(empty(s), ph, stop));
+      ok = __all_sync(0xffffffffu, mbar_wait(empty(s), ph, stop, a.wait_ns));
       if (!ok) break;
       const uint32_t sx = base + kWStage * s + q * kWX, sg = base + kWStage * s + 4 * 4 * kWX + q * kWG;
       int off[NX];
@@ -705,7 +723,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wgrad_tc_kernel(WgradTcArgs a, W
     for (int u = first; u < pl.bricks; u += pl.per) {
       int b, x0, y0, z0;
       brick(u, b, x0, y0, z0);
-      ok = __all_sync(0xffffffffu, mbar_wait(full(s), ph, stop));
+      ok = __all_sync(0xffffffffu, mbar_wait(full(s), ph, stop, a.wait_ns));
       if (!ok) break;
       fence_after();
       const int nk = min(kTY / 2, (g.H - y0 + 1) / 2);  // 16-voxel steps (two rows of y)
@@ -734,13 +752,10 @@ __global__ void __launch_bounds__(kWThreads, 1) wgrad_tc_kernel(WgradTcArgs a, W
     if (issue) mma_commit(done);
     __syncwarp();
   }
-  if (warp < 4 || (!ok && warp == kLoadWarps)) {
+  if (warp < 4) {
     // every MMA has finished (also after a failure, before TMEM is given back)
-    const unsigned long long t0 = now_ns();
-    bool fin = mbar_try(done, 0);
-    while (!fin && now_ns() - t0 < kWaitNs) fin = mbar_try(done, 0);
-    if (!fin) *stop = 1;
-    ok = __all_sync(0xffffffffu, fin && ok);
+    mbar_drain(done, 0, stop);
+    ok = __all_sync(0xffffffffu, mbar_try(done, 0) && ok);
   }
   if (warp < 4 && ok && first < pl.bricks) {
     fence_after();
@@ -769,7 +784,10 @@ __global__ void __launch_bounds__(kWThreads, 1) wgrad_tc_kernel(WgradTcArgs a, W
     fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTmemCols));
   }
-  if (tid == 0 && *stop) *reinterpret_cast<volatile int *>(a.err) = 1;
+  if (tid == 0 && *stop) {
+    *reinterpret_cast<volatile int *>(a.err) = 1;
+    *a.bad = 1;
+  }
 }
 
 // Tensor-core cycles of one plane that serves n output planes (per 16-channel

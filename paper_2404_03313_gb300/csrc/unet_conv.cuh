@@ -8,6 +8,8 @@ namespace s3ttv_net_detail {
 
 typedef __nv_bfloat16 bf16;
 
+constexpr unsigned long long kWaitNs = 4000000000ull;  // the waits' default time limit
+
 struct Vol {
   int B, D, H, W;
 };
@@ -34,7 +36,8 @@ struct ConvArgs {
   bf16 *y;            // [V][cout]
   int c0, c1, cout, relu;
   Vol g;
-  int *err;           // device-visible; set when a wait inside the kernel ran out
+  int *err, *bad;     // host and device memory; set when a wait inside the kernel ran out
+  unsigned long long wait_ns;  // time limit of such a wait (0: none is sat out)
   // With 32 output channels, optionally the network's head on the rounded outputs
   // f: h = Wh f + bh, (u, s, t) = (v + h0, h1, h2); hp holds Wh[3][32], then bh[3].
   // y may be null then: the layer's output is not stored.
@@ -58,7 +61,8 @@ struct WgradTcArgs {
   float *db;          // [cout]
   int c0, c1, cout;
   Vol vol;
-  int *err;
+  int *err, *bad;
+  unsigned long long wait_ns;
 };
 cudaError_t wgrad_prepare();
 cudaError_t wgrad_launch(const WgradTcArgs &a, int num_sms, cudaStream_t stream);
