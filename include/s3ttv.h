@@ -533,7 +533,8 @@ int s3ttv_net_gradient(s3ttv_net *net, const float *v, const float *u_ref, const
 
 /* One training step: the gradient as above, then one Adam update (beta1 0.9,
  * beta2 0.999, eps 1e-8, bias-corrected) with learning rate lr in [0, 1].
- * `loss` (may be NULL) receives the loss before the update. */
+ * `loss` (may be NULL) receives the loss before the update.  After an error in the
+ * gradient (S3TTV_ECUDA) the parameters and the Adam state are what they were. */
 int s3ttv_net_train_step(s3ttv_net *net, const float *v, const float *u_ref, const float *s_ref,
                          const float *t_ref, int B, int D, int H, int W, float lr, double *loss);
 

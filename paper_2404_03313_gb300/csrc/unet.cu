@@ -461,9 +461,11 @@ __global__ void __launch_bounds__(256) head_bwd_kernel(const bf16 *f, const floa
 }
 
 // ---------------------------------------------------------------- optimiser and weight packing
+// No step along a gradient that a kernel has given up on (bad).
 __global__ void adam_kernel(float *theta, const float *g, float *m, float *s, long long n, float lr, float b1,
-                            float b2, float eps, float c1, float c2) {
+                            float b2, float eps, float c1, float c2, const int *bad) {
   chained();
+  if (*bad) return;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const float gi = g[i];
     const float mi = fmaf(b1, m[i], (1.f - b1) * gi);
@@ -946,9 +948,10 @@ int s3ttv_net_train_step(s3ttv_net *net, const float *v, const float *u_ref, con
   const float c1 = (float)(1.0 / (1.0 - pow(b1, (double)net->adam_t)));
   const float c2 = (float)(1.0 / (1.0 - pow(b2, (double)net->adam_t)));
   NCU(launch_chained(adam_kernel, grid_for(net, net->tab.total, 256), 256, 0, net->stream, net->theta, net->grad,
-                     net->m1, net->m2, net->tab.total, lr, (float)b1, (float)b2, 1e-8f, c1, c2));
-  if ((rc = pack(net))) return rc;
-  return finish(net);
+                     net->m1, net->m2, net->tab.total, lr, (float)b1, (float)b2, 1e-8f, c1, c2, net->bad));
+  if (!(rc = pack(net))) rc = finish(net);
+  if (rc) net->adam_t -= 1;  // the step was not taken
+  return rc;
 }
 
 }  // extern "C"

@@ -58,3 +58,29 @@ def test_time_limit_is_checked(P):  # noqa: F811
             with pytest.raises(P.S3TTVError) as e:
                 net.set_option(key, value)
             assert e.value.status == P.EINVAL
+
+
+def test_no_training_step_along_a_failed_gradient(P):  # noqa: F811
+    """A step whose gradient fails leaves parameters, moments and step count alone: the
+    steps around it give what they give without it (they differ in the order of the
+    gradient's FP32 additions: 1e-3 of a step, as Adam divides a gradient by its size;
+    a step along the cut-off gradient moves parameters by 1e-3 = lr each)."""
+    args = volumes((2, 8, 8, 8))
+    runs = []
+    for fail in (False, True):
+        with P.WarmStartNet(0) as net:
+            net.set_params(bf16_params(23))
+            net.train_step(*args, 1e-3)
+            if fail:
+                before = net.get_params()
+                net.set_option(P.NET_OPT_WAIT_NS, 0)
+                with pytest.raises(P.S3TTVError) as e:
+                    net.train_step(*args, 1e-3)
+                assert e.value.status == P.ECUDA
+                net.set_option(P.NET_OPT_WAIT_NS, 4e9)
+                np.testing.assert_array_equal(net.get_params(), before)
+            loss = net.train_step(*args, 1e-3)
+            runs.append((loss, net.get_params()))
+    assert runs[0][0] == pytest.approx(runs[1][0], rel=1e-4)
+    moved = np.abs(runs[0][1] - runs[1][1])
+    assert np.mean(moved <= 1e-6) >= 0.99
