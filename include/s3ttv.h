@@ -381,8 +381,9 @@ int s3ttv_l1_ball(s3ttv_ctx *ctx, const float *x, float *out, long long n,
 int s3ttv_block_dual(s3ttv_ctx *ctx, float *Y, const float *ubar, float *Zv, float *Zh,
                      int N1, int N2, int N3, int k, float gamma_Y, s3ttv_info *info);
 
-/* The block-dual form S3TTV_OPT_AUTOTUNE chose: *tensor_cores 1 or 0 and
- * *ctas_per_sm (4 or 5), or *tensor_cores = -1 and *ctas_per_sm = 0 when none
+/* The block-dual form S3TTV_OPT_AUTOTUNE chose: *tensor_cores 0, 1 or 2 (as in
+ * S3TTV_OPT_TENSOR_CORES) and *ctas_per_sm (4 to 6, the CTAs per SM it is compiled
+ * for), or *tensor_cores = -1 and *ctas_per_sm = 0 when none
  * has been chosen.  Host pointers, required. */
 int s3ttv_tuned_form(const s3ttv_ctx *ctx, int *tensor_cores, int *ctas_per_sm);
 

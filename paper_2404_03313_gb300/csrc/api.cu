@@ -448,7 +448,7 @@ int block_dual_shape(s3ttv_ctx *ctx, const Dims &dm, int k, BdShape *sh) {
     return block_dual_variant_shape(ctx, dm, k, ctx->tuned_tc, ctx->tuned_minb, sh);
   }
   int per_sm = 0;
-  for (int minb = 5; minb >= 4; --minb) {
+  for (int minb = kMaxMinb; minb >= 4; --minb) {
     sh->v.minb = minb;
     if (!block_dual_has(sh->v)) continue;  // variant not compiled
     cudaError_t e = block_dual_prepare(sh->v, sh->smem);
@@ -1082,7 +1082,7 @@ int s3ttv_iterate(s3ttv_ctx *ctx, int n, float tol, s3ttv_info *info) {
     struct Cand { int tc, minb; BdShape sh; float ms = 1e30f; };
     std::vector<Cand> cands;
     for (int tc = 2; tc >= 0; --tc)
-      for (int minb = 5; minb >= 4; --minb) {
+      for (int minb = kMaxMinb; minb >= 4; --minb) {
         Cand c;
         c.tc = tc;
         c.minb = minb;

@@ -1730,10 +1730,10 @@ using KernelFn = void (*)(BlockDualArgs);
 // Variants compiled (null for the others): the CUDA-core form (tc 0) for 5
 // and 4 CTAs per SM; the tensor-core group form (tc 1) for 4 only (its five-
 // and six-CTA variants fit in shared memory, but at 96 and 80 registers they
-// spill and ran slower); the tensor-core streaming form (tc 2) for 4.
+// spill and ran slower); the tensor-core streaming form (tc 2) for stream_ctas(k).
 template <int K>
 KernelFn kernel_k(int minb, int tc) {
-  if (tc == 2) return minb == 4 ? block_dual_stream_kernel<K> : nullptr;
+  if (tc == 2) return minb == stream_ctas(K) ? block_dual_stream_kernel<K> : nullptr;
   if (tc) return minb == 4 ? block_dual_kernel<K, 4, true> : nullptr;
   if (minb != 5 && minb != 4) return nullptr;
   return minb == 5 ? block_dual_kernel<K, 5, false> : block_dual_kernel<K, 4, false>;

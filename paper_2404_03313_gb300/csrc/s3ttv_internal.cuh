@@ -167,9 +167,10 @@ size_t fallback_smem_bytes(int n);
 cudaError_t fallback_prepare(size_t smem_bytes);
 cudaError_t launch_fallback(const BlockDualArgs &a, int k, int stacked, int parts, int grid, size_t smem,
                             cudaStream_t st);
-// Kernel variant: block side k (1..5), minb = 5 or 4 (CTAs per SM its register
+// Kernel variant: block side k (1..5), minb = 4 to kMaxMinb (CTAs per SM its register
 // budget is sized for), tc = 1 for the Gram and the apply on tensor cores (three
-// TF32 products per FP32 product), 0 for FP32 CUDA cores.
+// TF32 products per FP32 product), 2 for its streaming form, 0 for FP32 CUDA cores.
+constexpr int kMaxMinb = 6;
 struct BdVariant {
   int k = 0;
   int minb = 4;
