@@ -154,13 +154,17 @@ __device__ __forceinline__ void store8(bf16 *p, const float f[8]) {
 }
 
 // ---------------------------------------------------------------- first layer's weight gradient
-// dW[o][j] = sum_p G[p, o] N[p, j] with N the 27 neighbour values of every voxel and a
-// one (im2col_first_kernel): 32 x 32 outputs over one chunk of voxels per CTA in
+// dW[o][j] = sum_p G[p, o] N[p, j] with N the 27 neighbour values of every voxel
+// (im2col_first_kernel): 32 x 32 outputs over one chunk of voxels per CTA in
 // stages of kWS, four warps of 16 x 16 (mma.sync; the other layers' weight gradients
-// run in unet_conv.cu).
+// run in unet_conv.cu).  The tensor cores' sums of kFold stages are added up in FP32
+// (they cut off what lies below a sum's last place, so its error grows with the number of
+// products added one after the other); the bias gradient is summed in FP32 by the threads
+// that copy G, with the rounding errors of its longer additions kept.
 constexpr int kAS = 40;     // shared row stride in bf16 (80 B: ldmatrix rows hit distinct banks)
 constexpr int kStages = 3;  // cp.async pipeline depth
 constexpr int kWS = 64;     // voxels per stage
+constexpr int kFold = 8;    // stages summed by the tensor cores at a time
 constexpr int kFirstSmem = kStages * kWS * 2 * kAS * (int)sizeof(bf16);
 
 __global__ void __launch_bounds__(128) wgrad_first_kernel(const bf16 *G, const bf16 *N, float *dw, float *db, int V,
@@ -185,11 +189,14 @@ __global__ void __launch_bounds__(128) wgrad_first_kernel(const bf16 *G, const b
       cp_async16(Xs + (buf * kWS + r) * kAS + q * 8, N + o, ok ? 16 : 0);
     }
   };
-  float acc[2][4];
+  float bs[8], bhi[8], blo[8];  // sums of this thread's pieces of G
+#pragma unroll
+  for (int i = 0; i < 8; ++i) bs[i] = bhi[i] = blo[i] = 0.f;
+  float acc[2][4], sum[2][4];  // the sums of kFold stages, of all
 #pragma unroll
   for (int j = 0; j < 2; ++j)
 #pragma unroll
-    for (int e = 0; e < 4; ++e) acc[j][e] = 0.f;
+    for (int e = 0; e < 4; ++e) acc[j][e] = sum[j][e] = 0.f;
 #pragma unroll
   for (int st = 0; st < kStages - 1; ++st) {
     if (st < nst) load(st, st);
@@ -202,6 +209,11 @@ __global__ void __launch_bounds__(128) wgrad_first_kernel(const bf16 *G, const b
     if (st + kStages - 1 < nst) load(st + kStages - 1, (st + kStages - 1) % kStages);
     cp_async_commit();
     const bf16 *gs = Gs + (st % kStages) * kWS * kAS, *xs = Xs + (st % kStages) * kWS * kAS;
+    float g0[8], g1[8];
+    load8(gs + r0 * kAS + q * 8, g0);
+    load8(gs + (r0 + 32) * kAS + q * 8, g1);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) bs[i] += g0[i] + g1[i];
 #pragma unroll
     for (int kk = 0; kk < kWS; kk += 16) {
       uint32_t af[4], bfr[4];  // A[m = out channel][k = voxel], B[k][n = neighbour], transposed on load
@@ -210,6 +222,22 @@ __global__ void __launch_bounds__(128) wgrad_first_kernel(const bf16 *G, const b
       mma_bf16(acc[0], af, bfr[0], bfr[1]);
       mma_bf16(acc[1], af, bfr[2], bfr[3]);
     }
+    if (st % kFold == kFold - 1 || st == nst - 1) {  // CTA-uniform
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          sum[j][e] += acc[j][e];
+          acc[j][e] = 0.f;
+        }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float x = bs[i], t = bhi[i] + x, b = t - bhi[i];
+        blo[i] += (bhi[i] - (t - b)) + (x - b);
+        bhi[i] = t;
+        bs[i] = 0.f;
+      }
+    }
   }
   const int gq = lane >> 2, t4 = lane & 3;
 #pragma unroll
@@ -217,8 +245,19 @@ __global__ void __launch_bounds__(128) wgrad_first_kernel(const bf16 *G, const b
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const int o = wm * 16 + gq + 8 * (e >> 1), c = wn * 16 + nj * 8 + 2 * t4 + (e & 1);
-      if (c <= 27) atomicAdd(c < 27 ? dw + o * 27 + c : db + o, acc[nj][e]);
+      if (c < 27) atomicAdd(dw + o * 27 + c, sum[nj][e]);
     }
+  float(*red)[32] = reinterpret_cast<float(*)[32]>(smem_raw);
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    float x = bhi[i] + blo[i];
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (lane < 4) red[warp][lane * 8 + i] = x;
+  }
+  __syncthreads();
+  if (tid < 32) atomicAdd(db + tid, (red[0][tid] + red[1][tid]) + (red[2][tid] + red[3][tid]));
 }
 
 // ---------------------------------------------------------------- first layer (one input channel)
@@ -284,9 +323,9 @@ __global__ void __launch_bounds__(256, 2) conv_first_kernel(const float *v, cons
   }
 }
 
-// col[p][j] = v[p + delta_j] for the 27 taps j (zero outside the volume), a one (so
-// that column 27 of the weight gradient is the bias gradient) and four zeros: the first layer's input as 32 BF16 channels, so its weight
-// gradient runs on the tensor-core weight-gradient kernel.
+// col[p][j] = v[p + delta_j] for the 27 taps j (zero outside the volume) and five zeros:
+// the first layer's input as 32 BF16 channels, so its weight gradient runs on the
+// tensor-core weight-gradient kernel.
 __global__ void __launch_bounds__(256) im2col_first_kernel(const float *v, bf16 *col, Vol g) {
   chained();
   const int V = nvox(g);
@@ -296,7 +335,7 @@ __global__ void __launch_bounds__(256) im2col_first_kernel(const float *v, bf16 
     float nb[32];
 #pragma unroll
     for (int t = 0; t < 32; ++t) {
-      nb[t] = t == 27 ? 1.f : 0.f;
+      nb[t] = 0.f;
       if (t < 27) {
         const int zz = z + t / 9 - 1, y2 = y + (t / 3) % 3 - 1, x2 = x + t % 3 - 1;
         if (zz >= 0 && zz < g.D && y2 >= 0 && y2 < g.H && x2 >= 0 && x2 < g.W)

@@ -575,34 +575,56 @@ __global__ void __launch_bounds__(kThreads, 1) conv_tc_kernel(ConvArgs a, Plan p
 // and 32 output channels per CTA: the voxels are the K dimension, so both operands
 // are read voxel-major (MN-major descriptors: a core matrix is 8 voxels of x by 8
 // channels, the layout of the forward kernel's planes).  M = 128 rows are the slice's
-// channels of the planes z - 1, z and z + 1 of X and a fourth plane whose first channel
-// is one everywhere; N = 32 are the output channels of plane z of G.  One tcgen05.mma
-// per 16 voxels thus covers the taps dz = -1, 0, +1 of one (dy, dx), and its row 96 sums
-// G: the bias gradient comes along.  The 27 x 32 x 32 gradients stay in TMEM, nine
-// accumulators of 32 columns, over all of a CTA's bricks (8 x 16 voxels of one plane),
-// and are then added into dW, 32 consecutive channels per instruction.
+// channels of the planes z - 1, z and z + 1 of X and a fourth plane of zeros; N = 32
+// are the output channels of plane z of G.  One tcgen05.mma per 16 voxels thus covers
+// the taps dz = -1, 0, +1 of one (dy, dx).  The 27 x 32 x 32 gradients stay in TMEM,
+// nine accumulators of 32 columns, over several of a CTA's bricks (8 x 16 voxels of one
+// plane), and are then added into dW, 32 consecutive channels per instruction.
+//
+// The tensor cores cut off what of a product lies below the running sum, so a sum's
+// error grows with the number of products added one after the other (WPlan::group).
+// The bias gradients are summed in FP32, a brick's values first and the bricks with the
+// additions' rounding errors kept: as a fourth plane of ones they came along with the
+// products, 3e-4 of themselves off (values of one sign, 256 x 256 x 128, 96 -> 32; now
+// 1e-7), and summed by the loading threads they held up the copies.
+// The largest error of a weight gradient of one sign there, with chains of a whole CTA's
+// bricks and now: 32 -> 32 1.2e-4, 4e-6; 96 -> 32 3.3e-4, 3e-6; 192 -> 64 2.1e-4, 1.1e-5
+// (with the mma.sync kernels 1.3e-4, 3.3e-4, 5.7e-5).
+//
 // Bound by the 40 cycles that M = 128, N = 32, K = 16 takes (its operand reads).  Against
 // the mma.sync kernels and column sums that it replaces (a tap per warp, every tap
 // gathering X again), four 32^3 crops, a layer with its bias gradient: 32 -> 32 at 32^3
 // 71 us before, 24 now; 96 -> 32 185 and 47; 192 -> 64 at 16^3 86 and 29; 64 -> 64 46 and 16
-// (the training gradient 1080 -> 690 us).
+// (the training gradient 1080 -> 690 us).  The issue of the MMAs keeps pace only without
+// divisions between them: with the bricks' rows known to be whole, the gradient at 256 x
+// 256 x 128 14.75 -> 14.26 ms.
 constexpr int kWX = (kPX * (kTY + 2) + 6) * 16;         // bytes of a plane's 8-channel piece of X (padded: 2 mod 8 pieces)
 constexpr int kWG = (kTX * kTY + 2) * 16;               // and of G
 constexpr int kWStage = 4 * 4 * kWX + 4 * kWG;
 constexpr int kWStages = 4;
-constexpr int kWThreads = (kLoadWarps + 1) * 32;        // 8 loading warps (the first four also write the result), 1 for the MMAs
+// 8 loading warps, 1 for the MMAs, 4 for the sums: one per quarter of the TMEM lanes, of
+// which the zero plane's sums G for the bias gradient
+constexpr int kWThreads = (kLoadWarps + 5) * 32;
 
 struct WPlan {
   int nsl, nt;         // slices of input channels, tiles of output channels
   int per;             // CTAs per (slice, tile)
   int tx, ty;          // bricks along x, y
   int bricks;
+  int group;           // bricks summed in TMEM before they are added into dW
 };
+
+// Add x into the sum hi + lo, keeping the rounding error in lo.
+__device__ __forceinline__ void two_sum(float &hi, float &lo, float x) {
+  const float s = hi + x, b = s - hi;
+  lo += (hi - (s - b)) + (x - b);
+  hi = s;
+}
 
 __global__ void __launch_bounds__(kWThreads, 1) wgrad_tc_kernel(WgradTcArgs a, WPlan pl) {
   chained();
   extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ __align__(8) uint64_t bars[2 * kWStages + 1];
+  __shared__ __align__(8) uint64_t bars[2 * kWStages + 3];
   __shared__ uint32_t s_tmem;
   __shared__ int s_stop;
   const int tid = threadIdx.x, lane = tid & 31;
@@ -613,7 +635,8 @@ __global__ void __launch_bounds__(kWThreads, 1) wgrad_tc_kernel(WgradTcArgs a, W
   const uint32_t base = smem_u32(smem), bar0 = smem_u32(bars);
   auto full = [&](int s) { return bar0 + 8u * s; };
   auto empty = [&](int s) { return bar0 + 8u * (kWStages + s); };
-  const uint32_t done = bar0 + 8u * (2 * kWStages);
+  // the accumulators hold a group's sums, have been read; all MMAs are done
+  const uint32_t acc_full = empty(kWStages), acc_empty = acc_full + 8, done = acc_full + 16;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&s_tmem)),
                  "r"(kTmemCols)
@@ -623,17 +646,18 @@ __global__ void __launch_bounds__(kWThreads, 1) wgrad_tc_kernel(WgradTcArgs a, W
   if (tid == kLoadWarps * 32) {
     for (int s = 0; s < kWStages; ++s) {
       mbar_init(full(s), kLoadWarps);
-      mbar_init(empty(s), 1);
+      mbar_init(empty(s), sl == 0 ? 2 : 1);  // the MMAs, the bias gradients
     }
+    mbar_init(acc_full, 1);
+    mbar_init(acc_empty, 3);
     mbar_init(done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     s_stop = a.wait_ns == 0;  // no wait is sat out
   }
-  // the fourth plane of every stage: channel 0 one, the others zero
+  // the fourth plane of every stage
   for (int i = tid; i < kWStages * 4 * (kWX / 16); i += kWThreads) {
     const int st = i / (4 * (kWX / 16)), e = i - st * 4 * (kWX / 16);
-    *reinterpret_cast<uint4 *>(smem + st * kWStage + 3 * 4 * kWX + e * 16) =
-        make_uint4(e < kWX / 16 ? 0x3f80u : 0u, 0u, 0u, 0u);
+    *reinterpret_cast<uint4 *>(smem + st * kWStage + 3 * 4 * kWX + e * 16) = make_uint4(0u, 0u, 0u, 0u);
   }
   asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
   fence_before();
@@ -641,6 +665,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wgrad_tc_kernel(WgradTcArgs a, W
   fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, s_tmem, 0);
   volatile int *stop = &s_stop;
+  const unsigned long long limit = a.wait_ns;
   auto brick = [&](int u, int &b, int &x0, int &y0, int &z0) {
     x0 = (u % pl.tx) * kTX;
     u /= pl.tx;
@@ -650,7 +675,6 @@ __global__ void __launch_bounds__(kWThreads, 1) wgrad_tc_kernel(WgradTcArgs a, W
     b = u / g.D;
   };
 
-  bool ok = true;
   if (warp < kLoadWarps) {
     // ---- brick copies: thread t keeps the 8-channel piece t mod 4 and steps over voxels ----
     constexpr int VS = kLoadWarps * 8, NVX = kPX * (kTY + 2), NX = (NVX + VS - 1) / VS, NG = kTX * kTY / VS;
@@ -670,8 +694,7 @@ __global__ void __launch_bounds__(kWThreads, 1) wgrad_tc_kernel(WgradTcArgs a, W
     for (int u = first; u < pl.bricks; u += pl.per) {
       int b, x0, y0, z0;
       brick(u, b, x0, y0, z0);
-      ok = __all_sync(0xffffffffu, mbar_wait(empty(s), ph, stop, a.wait_ns));
-      if (!ok) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(empty(s), ph, stop, limit))) break;
       const uint32_t sx = base + kWStage * s + q * kWX, sg = base + kWStage * s + 4 * 4 * kWX + q * kWG;
       int off[NX];
 #pragma unroll
@@ -711,76 +734,128 @@ __global__ void __launch_bounds__(kWThreads, 1) wgrad_tc_kernel(WgradTcArgs a, W
     }
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     if (prev >= 0) landed(prev);
-  } else {
+  } else if (warp == kLoadWarps) {
     // ---- MMA issue ----
     // F32 <- BF16 x BF16, A and B MN-major (bits 15, 16), N = 32, M = 128
     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | (4u << 17) | (8u << 24);
     // MN-major: the stride word is between 8-channel pieces, the leading word between 8-voxel groups of K
     const uint32_t ahi = desc_hi(kWX), bhi = desc_hi(kWG);
-    const bool issue = elect_one();
+    const bool issue = elect_one(), ragged = g.H % kTY != 0;
     int s = 0;
-    uint32_t ph = 0, add = 0;
-    for (int u = first; u < pl.bricks; u += pl.per) {
-      int b, x0, y0, z0;
-      brick(u, b, x0, y0, z0);
-      ok = __all_sync(0xffffffffu, mbar_wait(full(s), ph, stop, a.wait_ns));
-      if (!ok) break;
-      fence_after();
-      const int nk = min(kTY / 2, (g.H - y0 + 1) / 2);  // 16-voxel steps (two rows of y)
-      const uint32_t blo = uniform(desc_lo(base + kWStage * s + 4 * 4 * kWX, kTX * 16));
-      const uint32_t acc = uniform(add);
-      uint32_t tap = uniform(desc_lo(base + kWStage * s, kPX * 16)), d = tmem;
+    uint32_t ph = 0, gph = 1;  // gph: the parity of acc_empty that frees the accumulators for the group
+    bool ok = true;
+    // (a loop per group: bookkeeping in the loop over the bricks, where the issue of the
+    // MMAs bounds the kernel, cost 4% of it)
+    for (int u = first; u < pl.bricks && ok;) {
+      ok = __all_sync(0xffffffffu, mbar_wait(acc_empty, gph, stop, limit));
+      gph ^= 1;
+      uint32_t add = 0;
+      const int end = min(pl.bricks, u + pl.group * pl.per);
+      for (; u < end && ok; u += pl.per) {
+        // 16-voxel steps (two rows of y); no divisions where every brick is whole
+        int nk = kTY / 2;
+        if (ragged) nk = min(nk, (g.H - u / pl.tx % pl.ty * kTY + 1) / 2);
+        ok = __all_sync(0xffffffffu, mbar_wait(full(s), ph, stop, limit));
+        if (!ok) break;
+        fence_after();
+        const uint32_t blo = uniform(desc_lo(base + kWStage * s + 4 * 4 * kWX, kTX * 16));
+        const uint32_t acc = uniform(add);
+        uint32_t tap = uniform(desc_lo(base + kWStage * s, kPX * 16)), d = tmem;
 #pragma unroll 1
-      for (int yx = 0; yx < 9; ++yx) {
-        if (issue) {
+        for (int yx = 0; yx < 9; ++yx) {
+          if (issue) {
 #pragma unroll
-          for (int ks = 0; ks < kTY / 2; ++ks)
-            if (ks < nk) mma_f16(d, tap + ks * 2 * kPX, ahi, blo + ks * 2 * kTX, bhi, idesc, ks ? 1u : acc);
+            for (int ks = 0; ks < kTY / 2; ++ks)
+              if (ks < nk) mma_f16(d, tap + ks * 2 * kPX, ahi, blo + ks * 2 * kTX, bhi, idesc, ks ? 1u : acc);
+          }
+          __syncwarp();
+          tap += yx % 3 == 2 ? kPX - 2 : 1;
+          d += 32;
         }
+        add = 1;
+        if (issue) mma_commit(empty(s));
         __syncwarp();
-        tap += yx % 3 == 2 ? kPX - 2 : 1;
-        d += 32;
+        if (++s == kWStages) {
+          s = 0;
+          ph ^= 1;
+        }
       }
-      add = 1;
-      if (issue) mma_commit(empty(s));
-      __syncwarp();
-      if (++s == kWStages) {
-        s = 0;
-        ph ^= 1;
-      }
+      if (issue && ok) mma_commit(acc_full);
     }
     if (issue) mma_commit(done);
     __syncwarp();
-  }
-  if (warp < 4) {
-    // every MMA has finished (also after a failure, before TMEM is given back)
-    mbar_drain(done, 0, stop);
-    ok = __all_sync(0xffffffffu, mbar_try(done, 0) && ok);
-  }
-  if (warp < 4 && ok && first < pl.bricks) {
-    fence_after();
-    const uint32_t rows = tmem + ((uint32_t)(warp * 32) << 16);
-    uint32_t v[32];
-    if (warp < 3) {  // warp w holds tap plane dz = w - 1, a lane one input channel of the slice
-      const int cin = a.c0 + a.c1;
-      float *dst = a.dw + (size_t)(nt * 32) * 27 * cin + (size_t)(warp * 9) * cin + sl * 32 + lane;
+  } else if ((warp & 3) == 3) {
+    // ---- bias gradients: lane t sums the 8-channel piece t mod 4 of every 8th voxel ----
+    if (sl == 0) {
+      const int q = lane & 3, v0 = lane >> 2;
+      float hi[8], lo[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) hi[i] = lo[i] = 0.f;
+      int s = 0;
+      uint32_t ph = 0;
+      for (int u = first; u < pl.bricks; u += pl.per) {
+        if (!__all_sync(0xffffffffu, mbar_wait(full(s), ph, stop, limit))) break;
+        const unsigned char *sg = smem + kWStage * s + 4 * 4 * kWX + q * kWG + v0 * 16;
+        float x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = 0.f;
+#pragma unroll 8
+        for (int i = 0; i < kTX * kTY / 8; ++i) {
+          const uint4 w = *reinterpret_cast<const uint4 *>(sg + i * 128);
+          const uint32_t p[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {  // (a BF16 value is the upper half of its FP32 value)
+            x[2 * e] += __uint_as_float(p[e] << 16);
+            x[2 * e + 1] += __uint_as_float(p[e] & 0xffff0000u);
+          }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(empty(s));
+#pragma unroll
+        for (int i = 0; i < 8; ++i) two_sum(hi[i], lo[i], x[i]);
+        if (++s == kWStages) {
+          s = 0;
+          ph ^= 1;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        float x = hi[i] + lo[i];
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane < 4) atomicAdd(a.db + nt * 32 + lane * 8 + i, x);
+      }
+    }
+  } else {
+    // ---- a group's sums into dW: quarter w of the TMEM lanes holds tap plane dz = w - 1, a
+    // lane one input channel of the slice ----
+    const int w = warp & 3, cin = a.c0 + a.c1, nb = (pl.bricks - first + pl.per - 1) / pl.per;
+    const uint32_t rows = tmem + ((uint32_t)(w * 32) << 16);
+    float *dst = a.dw + (size_t)(nt * 32) * 27 * cin + (size_t)(w * 9) * cin + sl * 32 + lane;
+    uint32_t ph = 0;
+    for (int i = 0; i < nb; i += pl.group) {
+      if (!__all_sync(0xffffffffu, mbar_wait(acc_full, ph, stop, limit))) break;
+      ph ^= 1;
+      fence_after();
+#pragma unroll 3
       for (int yx = 0; yx < 9; ++yx) {
+        uint32_t v[32];
         tmem_ld32(v, rows + yx * 32);
+        if (yx == 8) {  // the next group's products may overwrite the accumulators
+          fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(acc_empty);
+        }
 #pragma unroll
         for (int o = 0; o < 32; ++o) atomicAdd(dst + ((size_t)o * 27 + yx) * cin, __uint_as_float(v[o]));
       }
-    } else if (sl == 0) {  // row 96: the sums of G
-      tmem_ld32(v, rows);
-      if (lane == 0)
-#pragma unroll
-        for (int o = 0; o < 32; ++o) atomicAdd(a.db + nt * 32 + o, __uint_as_float(v[o]));
     }
-    fence_before();
   }
   __syncwarp();
   fence_before();
   __syncthreads();
   if (warp == 0) {
+    if (*stop) mbar_drain(done, 0, stop);  // (otherwise the last sums read out say as much)
     fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(kTmemCols));
   }
@@ -901,6 +976,12 @@ cudaError_t wgrad_launch(const WgradTcArgs &a, int num_sms, cudaStream_t stream)
   pl.per = num_sms / (pl.nsl * pl.nt);
   if (pl.per < 1) pl.per = 1;
   if (pl.per > pl.bricks) pl.per = pl.bricks;
+  // Products added one after the other in TMEM: an eighth of a CTA's, but at least 192 and
+  // at most 1024 steps of 16 voxels (a group's end takes 3 us or so, 192 steps 33).
+  const int per_brick = a.vol.H < kTY ? (a.vol.H + 1) / 2 : kTY / 2;
+  const int own = (pl.bricks + pl.per - 1) / pl.per, steps = own * per_brick;
+  const int most = steps / 8 < 192 ? 192 : (steps / 8 > 1024 ? 1024 : steps / 8), groups = (steps + most - 1) / most;
+  pl.group = (own + groups - 1) / groups;
   return launch_chained(wgrad_tc_kernel, pl.nsl * pl.nt * pl.per, kWThreads, kWStages * kWStage, stream, a, pl);
 }
 
