@@ -8,6 +8,8 @@ rounding) and of the FP32 additions into Z of the block regularisers (k^2 = 4
 terms, 4 u relative), over a few dozen passes: 1e-5 relative L2.  A dual step that
 runs on past the stop moves Y by more than 1e-2.
 """
+import time
+
 import numpy as np
 import pytest
 
@@ -56,3 +58,27 @@ def test_state_after_the_stop_does_not_depend_on_check_every(P, reg):
         for n in one:
             err = np.linalg.norm(one[n].astype(np.float64) - many[n]) / max(np.linalg.norm(one[n]), 1e-30)
             assert err <= TOL, (n, err)
+
+
+def test_passes_beyond_the_stop_leave_the_memory_alone(P):
+    """Passes enqueued beyond the stop cost their launches, whatever the size of the cube
+    (they come with every batch whose members stop at different passes): 400 of them take
+    no more than twice the time on 64 MB cubes than on 64 KB ones, plus 2 ms.  A kernel that
+    goes on over the cubes takes 40 us of each."""
+    seconds = {}
+    for shape in ((32, 32, 16), (256, 256, 256)):
+        v = torch.rand(shape, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+        n = v.numel()
+        best = []
+        with P.Solver(0) as s:
+            s.set_option(P.OPT_CHECK_EVERY, 400)
+            s.setup(v, 0.05 * n ** 0.5, 0.02 * n, 0.02 * n, 1)
+            s.iterate(2)
+            for _ in range(3):
+                t0 = time.perf_counter()
+                assert s.iterate(400, 1e6)["iters"] == 1  # any change is below this tolerance
+                best.append(time.perf_counter() - t0)
+        seconds[shape] = min(best)
+    small, large = seconds.values()
+    print(f"400 passes, one before the stop: {1e3 * small:.2f} ms, {1e3 * large:.2f} ms")
+    assert large <= 2 * small + 2e-3, seconds
