@@ -561,7 +561,7 @@ cudaError_t launch_Y_to_external(const float *in, float *ext, Dims dm, int k, cu
 
 cudaError_t launch_xfield(const float *ubar, float *Fv, float *Fh, Dims dm, int grid, cudaStream_t st, int open_s,
                           int first_order, float *Fs, const L1Args *l1) {
-  const int nh = l1 ? grid / 2 : 0;  // (grid: two CTAs per SM)
+  const int nh = l1 ? (grid + 1) / 2 : 0;  // (grid: two CTAs per SM; a grid of one still takes both thresholds)
   return launch_chained(xfield_kernel, grid + 2 * nh, kSelThreads, 0, st, ubar, Fv, Fh, dm, open_s, first_order, Fs,
                         l1 ? *l1 : L1Args(), nh);
 }
