@@ -54,9 +54,10 @@ constexpr int kCW = 48;        // columns of Y' per streamed chunk
 // The Gram's 4 x 4 tiles read four chunk rows apart (4 (kCW + 4) floats, 16
 // banks mod 32) and rotate their column order within 16-column windows.
 static_assert(kCW % 16 == 0 && (4 * (kCW + 4)) % 32 == 16, "chunk geometry of the Gram's bank rotation");
-// Lanes per row pair in the Jacobi: 8, or 4 where that lets one round of the
-// CTA's warps cover every pair of a step (n / 2 pairs) and 8 would need more;
-// blocks above kMaxSmemRows rows always 8 (at most 32 floats of a row per lane).
+// Lanes per row pair: 8, or 4 where that lets one round of the CTA's warps cover
+// every pair of a step (n / 2 pairs) and 8 would need more.  The Jacobi meets two rows
+// only in blocks of 37..63 rows (use_quads()); above kMaxSmemRows rows the value sets
+// the row stride of the matrices in global memory, elsewhere nothing.
 __host__ __device__ constexpr int pair_lanes(int n, int lw) {
   return n > kMaxSmemRows ? 8
                           : (((n + 1) / 2 + lw * 8 - 1) / (lw * 8) < ((n + 1) / 2 + lw * 4 - 1) / (lw * 4) ? 4 : 8);

@@ -4,10 +4,11 @@
 
 namespace s3ttv {
 
-// The kernels are launched as programmatic dependents of one another: chained() is the first statement of each, lets the next kernel's CTAs come in as
-// soon as this one's have all started, and waits for the kernel before to be done
-// (with its writes), so launch latency and CTA set-up overlap the tail of the
-// kernel before.  No kernel touches memory ahead of it.
+// The kernels are launched as programmatic dependents of one another: chained() is
+// the first statement of each, lets the next kernel's CTAs come in as soon as this
+// one's have all started, and waits for the kernel before to be done (with its
+// writes), so launch latency and CTA set-up overlap the tail of the kernel before.
+// No kernel touches memory ahead of it.
 __device__ __forceinline__ void chained() {
   asm volatile("griddepcontrol.launch_dependents;\n griddepcontrol.wait;\n" ::: "memory");
 }
