@@ -62,7 +62,7 @@ FALLBACK_HBM_GBS = 6800.0
 # form), from an ncu capture of the kernel whose source hashes to `sha`
 # (profiles/block_dual_stream_k5_128x128x128.md); traffic is reported only
 # while the kernel source is unchanged.
-BLOCK_DUAL_TRAFFIC = {"sha": "31fd0bbe11388b09", "k": 5, "bytes_per_voxel": (535.600128e6 + 518.705664e6) / 2097152}
+BLOCK_DUAL_TRAFFIC = {"sha": "479aae58f9201275", "k": 5, "bytes_per_voxel": (533.152768e6 + 516.918784e6) / 2097152}
 
 
 # ---------------------------------------------------------------------------

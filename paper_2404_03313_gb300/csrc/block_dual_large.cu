@@ -595,8 +595,9 @@ __global__ void __launch_bounds__(large_warps<K, ST, PARTS>() * 32, large_ctas(S
       // order, and a group of QL lanes holds the four rows of a meeting in
       // registers and rotates the four row pairs across it (at a sweep's first
       // step also the two within).  Against one row pair per meeting this halves
-      // the rows loaded and stored, which bound the sweep (62k of 96k cycles per
-      // sweep and SM at n = 100 were shared-memory wavefronts), and the barriers.
+      // the rows loaded and stored, which bound the sweep, and the barriers (blocks of
+      // 100 rows by 128 columns: 256 k shared-memory wavefronts each, 66% of their
+      // peak, before; 175 k, 48%, with two row pairs).
       for (int step = 0; step < NS - 1; ++step) {
         for (int base = 0; base < NS / 2; base += LW * (32 / QL)) {
           if (base + warp * (32 / QL) >= NS / 2) continue;  // the whole warp has no quad this round
