@@ -336,17 +336,18 @@ __global__ void Z_from_Y_kernel(const float *__restrict__ Y, float *__restrict__
 // Fv = D_v D_s ubar and Fh = D_h D_s ubar: the second-order differences the
 // structure tensors of eq. (SSST) are cut from, formed once per pass.
 // The first 2 nh CTAs take the second level of the l1-ball thresholds of s and t
-// instead (independent of F): one launch for both.  In a pass (nh > 0) nothing is read
+// instead (independent of F): one launch for both.  In a pass (nh > 0) it ends at once
 // once the stop rule has fired: in a batch, stopped members go on until all have.
 __global__ void __launch_bounds__(kSelThreads, 3) xfield_kernel(const float *__restrict__ ubar, float *__restrict__ Fv,
                                                                 float *__restrict__ Fh, Dims dm, int open_s,
                                                                 int first_order, float *__restrict__ Fs, L1Args l1,
                                                                 int nh) {
   chained();
-  if (nh > 0 && l1.sc->done) return;
+  const int done = nh > 0 ? l1.sc->done : 0;
   if ((int)blockIdx.x < 2 * nh) {
     __shared__ BinSums s_hist;
     const int pb = (int)blockIdx.x >= nh, cta = blockIdx.x - pb * nh;
+    if (done) return;
     const L1State st = l1.sc->l1[pb];
     if (st.mode != 0) return;  // decided at the first level
     l1_hist<2, true>(l1, st, pb, (long long)cta * kSelThreads + threadIdx.x, (long long)nh * kSelThreads, s_hist);
@@ -385,6 +386,7 @@ __global__ void __launch_bounds__(kSelThreads, 3) xfield_kernel(const float *__r
         fv[e] = fh[e] = 0.f;
       }
     }
+    if (done) return;  // (looked at here, the flag's latency hides behind the first loads)
     st4(Fv + p0 + b0, make_float4(fv[0], fv[1], fv[2], fv[3]));
     st4(Fh + p0 + b0, make_float4(fh[0], fh[1], fh[2], fh[3]));
     if (Fs) st4(Fs + p0 + b0, make_float4(fs[0], fs[1], fs[2], fs[3]));
