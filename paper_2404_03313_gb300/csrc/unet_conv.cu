@@ -107,6 +107,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   if (mbar_try(bar, parity)) return true;
   const unsigned long long t0 = now_ns();
   while (true) {
+#pragma unroll 1  // (unrolled into every role's loops, the tries crowd the instruction cache)
     for (int i = 0; i < 32; ++i)
       if (mbar_try(bar, parity)) return true;
     if (*stop) return false;
