@@ -336,24 +336,25 @@ __global__ void Z_from_Y_kernel(const float *__restrict__ Y, float *__restrict__
 // Fv = D_v D_s ubar and Fh = D_h D_s ubar: the second-order differences the
 // structure tensors of eq. (SSST) are cut from, formed once per pass.
 // The first 2 nh CTAs take the second level of the l1-ball thresholds of s and t
-// instead (independent of F): one launch for both.  In a pass (nh > 0) it ends at once
-// once the stop rule has fired: in a batch, stopped members go on until all have.
+// instead (independent of F): one launch for both.
+// stop: null, or where the others look whether the stop rule has fired (in a batch,
+// stopped members go on until all have).
 __global__ void __launch_bounds__(kSelThreads, 3) xfield_kernel(const float *__restrict__ ubar, float *__restrict__ Fv,
                                                                 float *__restrict__ Fh, Dims dm, int open_s,
                                                                 int first_order, float *__restrict__ Fs, L1Args l1,
-                                                                int nh) {
+                                                                int nh, const Scalars *stop) {
   chained();
-  const int done = nh > 0 ? l1.sc->done : 0;
   if ((int)blockIdx.x < 2 * nh) {
     __shared__ BinSums s_hist;
     const int pb = (int)blockIdx.x >= nh, cta = blockIdx.x - pb * nh;
-    if (done) return;
+    if (l1.sc->done) return;
     const L1State st = l1.sc->l1[pb];
     if (st.mode != 0) return;  // decided at the first level
     l1_hist<2, true>(l1, st, pb, (long long)cta * kSelThreads + threadIdx.x, (long long)nh * kSelThreads, s_hist);
     if (last_cta(&l1.sc->ticket[pb], nh)) l1_scan_level<2>(l1, pb);
     return;
   }
+  if (stop && stop->done) return;
   const int first = (blockIdx.x - 2 * nh) * blockDim.x + threadIdx.x, stride = (gridDim.x - 2 * nh) * blockDim.x;
   const int N3p = dm.N3p, C4 = N3p >> 2, N2 = dm.N2;
   const int nch = (int)(dm.P * C4);
@@ -386,7 +387,6 @@ __global__ void __launch_bounds__(kSelThreads, 3) xfield_kernel(const float *__r
         fv[e] = fh[e] = 0.f;
       }
     }
-    if (done) return;  // (looked at here, the flag's latency hides behind the first loads)
     st4(Fv + p0 + b0, make_float4(fv[0], fv[1], fv[2], fv[3]));
     st4(Fh + p0 + b0, make_float4(fh[0], fh[1], fh[2], fh[3]));
     if (Fs) st4(Fs + p0 + b0, make_float4(fs[0], fs[1], fs[2], fs[3]));
@@ -564,8 +564,12 @@ cudaError_t launch_Y_to_external(const float *in, float *ext, Dims dm, int k, cu
 cudaError_t launch_xfield(const float *ubar, float *Fv, float *Fh, Dims dm, int grid, cudaStream_t st, int open_s,
                           int first_order, float *Fs, const L1Args *l1) {
   const int nh = l1 ? (grid + 1) / 2 : 0;  // (grid: two CTAs per SM; a grid of one still takes both thresholds)
+  // F of a stopped problem is left alone from 8 chunks a thread on (4 M voxels or so, which
+  // the L2 does not hold for long); below, looking at the flag costs more than it saves
+  // (32 x 32 x 16: 0.25 us of 44 in every pass)
+  const Scalars *stop = l1 && dm.Np / 4 >= 8LL * grid * kSelThreads ? l1->sc : nullptr;
   return launch_chained(xfield_kernel, grid + 2 * nh, kSelThreads, 0, st, ubar, Fv, Fh, dm, open_s, first_order, Fs,
-                        l1 ? *l1 : L1Args(), nh);
+                        l1 ? *l1 : L1Args(), nh, stop);
 }
 
 cudaError_t launch_Z_from_Y(const float *Y, float *Zv, float *Zh, Dims dm, int k, cudaStream_t st, float *Zs) {
